@@ -228,11 +228,9 @@ wfq_status_t wfq_prepare_filters(wfq_plan_t *plan, const float *w_dev, const flo
  * whose memory pool owns the whole device, a real-time loop where the allocator's
  * implicit device synchronisation is not acceptable, or a process whose device memory
  * was fully budgeted at start-up.  This call produces the same codes and scales as
- * wfq_prepare_filters (same kernels, same arithmetic) and allocates nothing: no
- * cudaMalloc/cudaFree, no host allocation, no library routine that allocates.  The fp32
- * transformed filters it needs between its two kernels are kept in one array that is
- * part of the library's device image, WFQ_STATIC_SCRATCH_FLOATS floats (16 MiB); every
- * GPU on which the library is loaded holds that array until the process exits.
+ * wfq_prepare_filters (same kernel, same arithmetic) and allocates nothing: no
+ * cudaMalloc/cudaFree, no host allocation, no library routine that allocates, and no
+ * scratch of its own.
  *
  *   w_dev        device, fp32 [K][C][3][3]                               (input)
  *   sG_host      host, m+2 floats, diagonal of S_G; NULL = standard scales
@@ -244,14 +242,7 @@ wfq_status_t wfq_prepare_filters(wfq_plan_t *plan, const float *w_dev, const flo
  * WFQ_ERR_SCRATCH_TOO_SMALL is returned and nothing is launched.  Other argument errors
  * are reported as in wfq_prepare_filters.  Asynchronous on `stream`.
  *
- * The first call on each device looks up the device address of the built-in array
- * (with that device current); make that first call outside any stream capture.  All
- * calls on a device share the one array: it still holds the previous call's values
- * when a call starts (harmless, every element that is read is written first by the
- * same call, so nothing needs clearing), and two calls whose kernels can overlap on
- * the GPU (different streams, or different host threads) race on it.  Serialise them.
- * The looked-up address is cached per device ordinal for the life of the process;
- * cudaDeviceReset invalidates it, so do not call this function after a device reset.
+ * Calls share nothing: they may overlap on different streams and from different threads.
  */
 #define WFQ_STATIC_SCRATCH_FLOATS (4u * 1024u * 1024u)
 wfq_status_t wfq_quantize_filters_static(const float *w_dev, int K, int C, int m, int group_size,

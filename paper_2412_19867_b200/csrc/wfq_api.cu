@@ -352,17 +352,7 @@ wfq_status_t wfq_prepare_filters(wfq_plan_t *plan, const float *w_dev, const flo
 
     wfq_status_t bs = ensure_filter_buffers(plan, as_stream(stream));
     if (bs != WFQ_OK) return bs;
-    cudaError_t e;
-    const size_t wq_bytes = (size_t)g.P * g.K * g.C;
-    // fp32 transformed filters between the two kernels: stream-ordered allocation, released
-    // in stream order after the quantization kernel, so the call neither blocks nor holds
-    // the temporary (four times the size of Wq) any longer than the kernels need it
-    void *w32 = nullptr;
-    if ((e = cudaMallocAsync(&w32, wq_bytes * sizeof(float), as_stream(stream))) != cudaSuccess)
-        return cuda_status(e);
-    e = wfq::launch_filter_prep(*plan, w_dev, static_cast<float *>(w32), as_stream(stream));
-    cudaError_t e2 = cudaFreeAsync(w32, as_stream(stream));
-    if (e != cudaSuccess || e2 != cudaSuccess) return WFQ_ERR_CUDA;
+    if (wfq::launch_filter_prep(*plan, w_dev, as_stream(stream)) != cudaSuccess) return WFQ_ERR_CUDA;
     return finish_filters(plan);
 }
 

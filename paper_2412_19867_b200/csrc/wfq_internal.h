@@ -163,8 +163,7 @@ namespace wfq {
 
 // Kernel launchers (one per translation unit).  Each returns a cudaError_t from the
 // launch; none synchronises.
-cudaError_t launch_filter_prep(const wfq_plan &plan, const float *w_dev, float *scratch_w32,
-                               cudaStream_t stream);
+cudaError_t launch_filter_prep(const wfq_plan &plan, const float *w_dev, cudaStream_t stream);
 // 4-bit filter codes <-> two codes per byte (the exported blob's storage); n_codes a multiple of 8
 cudaError_t launch_pack_nibbles(const int8_t *codes, void *packed, size_t n_codes, cudaStream_t stream);
 cudaError_t launch_unpack_nibbles(const void *packed, int8_t *codes, size_t n_codes, cudaStream_t stream);
