@@ -177,7 +177,7 @@ wfq_status_t wfq_plan_set_weight_bits(wfq_plan_t *plan, int bits);
  * With an integer output transform the scale vectors given to wfq_prepare_filters change the
  * result (this is where the paper's learned scales act); with the floating-point transforms they
  * are numerically neutral.  Group sizes: multiples of 32 up to 256.  Host only; takes effect from
- * the next forward call.  These kernels are reference-speed implementations.
+ * the next forward call.
  */
 typedef enum { WFQ_Y_FP32 = 0, WFQ_Y_TILE = 1, WFQ_Y_ROW = 2 } wfq_y_quant_t;
 wfq_status_t wfq_plan_set_full_quant(wfq_plan_t *plan, int quant_input, wfq_y_quant_t y_mode);

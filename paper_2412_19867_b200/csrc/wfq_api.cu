@@ -62,7 +62,7 @@ wfq_status_t bind_device(wfq_plan *plan)
         if (!g_device_ready[dev]) {
             if (wfq::setup_input_transform() != cudaSuccess || wfq::setup_input_transform_tc() != cudaSuccess ||
                 wfq::setup_gemm() != cudaSuccess || wfq::setup_output_transform() != cudaSuccess ||
-                wfq::setup_full_quant() != cudaSuccess || wfq::setup_input_transform_tcn() != cudaSuccess)
+                wfq::setup_input_transform_tcn() != cudaSuccess)
                 return WFQ_ERR_CUDA;
             g_device_ready[dev] = true;
         }
@@ -499,7 +499,7 @@ wfq_status_t wfq_output_transform(wfq_plan_t *plan, float *y_dev, void *stream)
     wfq_status_t s = ready_to_run(plan);
     if (s != WFQ_OK) return s;
     if (!y_dev || (reinterpret_cast<uintptr_t>(y_dev) & 15u)) return WFQ_ERR_INVALID_ARG;
-    if (plan->fq_output) return cuda_status(wfq::launch_output_transform_int(*plan, y_dev, as_stream(stream)));
+    if (plan->fq_output) return cuda_status(wfq::launch_output_transform_int(*plan, y_dev, as_stream(stream), false));
     return cuda_status(wfq::launch_output_transform(*plan, y_dev, as_stream(stream), false));
 }
 
@@ -515,7 +515,7 @@ wfq_status_t wfq_conv_forward(wfq_plan_t *plan, const void *x_dev, float *y_dev,
                                    : wfq::launch_input_transform(*plan, x_dev, st);
     if (e == cudaSuccess) e = wfq::launch_gemm(*plan, nullptr, st, true);
     if (e == cudaSuccess)
-        e = plan->fq_output ? wfq::launch_output_transform_int(*plan, y_dev, st)
+        e = plan->fq_output ? wfq::launch_output_transform_int(*plan, y_dev, st, true)
                             : wfq::launch_output_transform(*plan, y_dev, st, true);
     return cuda_status(e);
 }

@@ -26,6 +26,7 @@
 // the group in registers.
 #include <cuda_fp16.h>
 
+#include "wfq_int_quant.cuh"
 #include "wfq_internal.h"
 #include "wfq_ptx.cuh"
 
@@ -392,7 +393,7 @@ __device__ __forceinline__ void group_scale(float amax, float &scale, float &inv
 // ---- phase 2 of a work item: quantize, one (tile, group, position) per thread -------------
 // Zs holds the transformed values of `ntile` tiles as [tile][position][CB + 4] fp32; the item is
 // tiles tw0 .. of tile row `srow` (= image * TH + tile row) and channels c_base .. c_base + CB.
-template <int P, int GSR, int SPLIT>
+template <int P, int GSR, int SPLIT, bool SCALED = true>
 __device__ __forceinline__ void quantize_item(const float *__restrict__ Zs, int CBP, int ntile, int ng, int gs,
                                               int srow, int tw0, int c_base, const Geometry &g,
                                               const ScaleTables &tab, int8_t *__restrict__ Xq,
@@ -421,7 +422,7 @@ __device__ __forceinline__ void quantize_item(const float *__restrict__ Zs, int 
             float amax = 0.f;
 #pragma unroll
             for (int k = 0; k < GSR / 4; ++k) {
-                v[k] = scale4(src[k], sp2, sl2);
+                v[k] = SCALED ? scale4(src[k], sp2, sl2) : src[k];
                 amax = absmax4(amax, v[k]);
             }
             if constexpr (SPLIT >= 2) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 1));
@@ -448,19 +449,20 @@ __device__ __forceinline__ void quantize_item(const float *__restrict__ Zs, int 
             int8_t *dst = Xq + ((size_t)p * g.T + t) * g.C + c_base + grp * gs;
             const float sp = tab.in_scale[p], sl = tab.in_scale_lo[p];
             const float2 sp2 = make_float2(sp, sp), sl2 = make_float2(sl, sl);
+            auto val = [&](int k) { return SCALED ? scale4(src[k], sp2, sl2) : src[k]; };
             float scale, inv;
             float amax = 0.f;
-            for (int k = 0; k < gs / 4; ++k) amax = absmax4(amax, scale4(src[k], sp2, sl2));
+            for (int k = 0; k < gs / 4; ++k) amax = absmax4(amax, val(k));
             group_scale(amax, scale, inv);
             for (int k = 0; k < gs / 32; ++k)
-                st_global_v8_b32(dst + 32 * k, codes4(scale4(src[8 * k], sp2, sl2), inv),
-                                 codes4(scale4(src[8 * k + 1], sp2, sl2), inv), codes4(scale4(src[8 * k + 2], sp2, sl2), inv),
-                                 codes4(scale4(src[8 * k + 3], sp2, sl2), inv), codes4(scale4(src[8 * k + 4], sp2, sl2), inv),
-                                 codes4(scale4(src[8 * k + 5], sp2, sl2), inv), codes4(scale4(src[8 * k + 6], sp2, sl2), inv),
-                                 codes4(scale4(src[8 * k + 7], sp2, sl2), inv));
+                st_global_v8_b32(dst + 32 * k, codes4(val(8 * k), inv), codes4(val(8 * k + 1), inv),
+                                 codes4(val(8 * k + 2), inv), codes4(val(8 * k + 3), inv),
+                                 codes4(val(8 * k + 4), inv), codes4(val(8 * k + 5), inv),
+                                 codes4(val(8 * k + 6), inv), codes4(val(8 * k + 7), inv));
             sX[((size_t)p * g.G + g_base + grp) * g.Ts + t] = scale;
         }
-    }}
+    }
+}
 
 // ---- the kernel ----------------------------------------------------------------------
 // GSR > 0: channels a thread holds in registers during phase 2 (32 or 64); a group is GSR *
@@ -546,6 +548,128 @@ input_transform_kernel(const Tin *__restrict__ x, int8_t *__restrict__ Xq,
         if (!prm.dbuf && next < prm.items) stage_item(next, 0);   // the strip buffer is free: refill it now
 
         quantize_item<P, GSR, SPLIT>(Zs, CBP, ntile, ng, gs, srow, tw0, c_base, g, tab, Xq, sX);
+        __syncthreads();   // Z and this strip buffer are free again
+    }
+}
+
+// ---- the fully quantized input transform (Eq. quant-B) ------------------------------------
+//   X~ = s_qB^2 s_qx  Q(S_B V_B / s_qB)  Q(x / s_qx)  Q(V_B^T S_B / s_qB)
+// with one s_qx per (tile, channel group) over the group's n x n patches; fp32(X~) is what the group
+// quantizer of the contraction's operand sees.  Work items, staging and quantization are those of
+// the kernel above; in between every (tile, channel) first contributes its patch to the abs-max of its
+// 32 channels (one warp reduction), then quantizes the patch (code_of_float) and forms the two
+// integer products.  32x32 C=640 F(4,3), two images: 15.5 us (latency of
+// the phases at 16 warps per SM, 45 % of the issue slots); with one CTA per (tile, group), each thread
+// reading its patch element by element from global memory (32 rows of memory per load instruction)
+// and all codes decided in fp64, 24.8 us.
+template <int M, typename Tin, int GSR, int SPLIT>
+__global__ void __launch_bounds__(K1_THREADS, 4)
+input_transform_int_kernel(const Tin *__restrict__ x, int8_t *__restrict__ Xq, float *__restrict__ sX, Geometry g,
+                           const __grid_constant__ FullQuantTables tab, K1Params prm)
+{
+    constexpr int NN = M + 2;
+    constexpr int P = NN * NN;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ float amax_s[(K1_WP - 3) / M][8];               // [tile][run of 32 channels]
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    float *Zs = reinterpret_cast<float *>(smem_raw + (1 + prm.dbuf) * prm.strip_bytes);   // [tile][position][CBP]
+    const int CBP = prm.CB + 4;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr int NWARP = K1_THREADS / 32;
+    const int cb32 = prm.CB >> 5;
+    const int gs = GSR > 0 ? GSR * SPLIT : g.gs;
+    const int ng = prm.CB / gs, gs32 = gs >> 5;
+
+    auto stage_item = [&](int item, int buf) {
+        const int cblk = item % prm.NCB, rest = item / prm.NCB;
+        const int srow = rest / prm.NCH, chunk = rest - srow * prm.NCH;
+        const int img = srow / g.TH, th = srow - img * g.TH;
+        const int first = chunk * prm.TB * M - 1;
+        const int w_base = prm.vec16 ? ((first + 8) & ~7) - 8 : first - 1;
+        stage_strip<Tin, NN>(reinterpret_cast<Tin *>(smem_raw + buf * prm.strip_bytes), x, g, prm, img,
+                             cblk * prm.CB, th * M - 1, w_base);
+        cp_async_commit();
+    };
+
+    int item = blockIdx.x;
+    if (prm.dbuf && item < prm.items) stage_item(item, 0);
+    for (int it = 0; item < prm.items; ++it, item += gridDim.x) {
+        const int buf = prm.dbuf ? (it & 1) : 0;
+        const int next = item + gridDim.x;
+        if (!prm.dbuf) {
+            if (it == 0) stage_item(item, 0);
+            cp_async_wait_group<0>();
+        } else if (next < prm.items) {
+            stage_item(next, buf ^ 1);
+            cp_async_wait_group<1>();
+        } else {
+            cp_async_wait_group<0>();
+        }
+        __syncthreads();
+
+        const Tin *strip = reinterpret_cast<const Tin *>(smem_raw + buf * prm.strip_bytes);
+        const int cblk = item % prm.NCB, rest = item / prm.NCB;
+        const int srow = rest / prm.NCH, chunk = rest - srow * prm.NCH;   // srow = img*TH + th
+        const int tw0 = chunk * prm.TB;
+        const int ntile = min(prm.TB, g.TW - tw0);
+        const int c_base = cblk * prm.CB;
+        const int voff = tw0 * M - 2 - (((tw0 * M - 1 + 8) & ~7) - 8);
+        auto patch = [&](int tl, int c, float (&d)[NN][NN]) {
+            if (sizeof(Tin) == 2 && prm.vec16) load_patch_vec<NN>(strip + c * prm.CS, tl * M + voff, d);
+            else load_patch<NN>(strip + c * prm.CS, tl * M, d);
+        };
+
+        for (int wt = warp; wt < ntile * cb32; wt += NWARP) {
+            const int tl = wt / cb32, c32 = wt - tl * cb32;
+            float d[NN][NN], m = 0.f;
+            patch(tl, c32 * 32 + lane, d);
+#pragma unroll
+            for (int a = 0; a < NN; ++a)
+#pragma unroll
+                for (int b = 0; b < NN; ++b) m = fmaxf(m, fabsf(d[a][b]));     // ignores NaN
+            const unsigned top = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+            if (lane == 0) amax_s[tl][c32] = __uint_as_float(top);
+        }
+        __syncthreads();
+        for (int wt = warp; wt < ntile * cb32; wt += NWARP) {
+            const int tl = wt / cb32, c32 = wt - tl * cb32;
+            const int c = c32 * 32 + lane;
+            float amax = 0.f;                                    // of the group of these 32 channels
+            for (int k = c32 / gs32 * gs32, e = k + gs32; k < e; ++k) amax = fmaxf(amax, amax_s[tl][k]);
+            float d[NN][NN];
+            patch(tl, c, d);
+            const float rinv = __fdiv_rn(127.f, amax);
+            int q[NN][NN], tmp[NN][NN];
+#pragma unroll
+            for (int a = 0; a < NN; ++a)
+#pragma unroll
+                for (int b = 0; b < NN; ++b) q[a][b] = code_of_float(d[a][b], amax, rinv);
+#pragma unroll
+            for (int b = 0; b < NN; ++b)
+#pragma unroll
+                for (int i = 0; i < NN; ++i) {
+                    int s = 0;
+#pragma unroll
+                    for (int a = 0; a < NN; ++a) s += tab.BTq[i * NN + a] * q[a][b];
+                    tmp[i][b] = s;
+                }
+            const double scale = __dmul_rn(tab.sqB2, __ddiv_rn((double)amax, kIntQmax));
+            float *out = Zs + (size_t)tl * P * CBP + c;
+#pragma unroll
+            for (int i = 0; i < NN; ++i)
+#pragma unroll
+                for (int j = 0; j < NN; ++j) {
+                    int s = 0;
+#pragma unroll
+                    for (int b = 0; b < NN; ++b) s += tmp[i][b] * tab.BTq[j * NN + b];
+                    out[(i * NN + j) * CBP] = (float)__dmul_rn((double)s, scale);
+                }
+        }
+        __syncthreads();
+        if (!prm.dbuf && next < prm.items) stage_item(next, 0);   // the strip buffer is free: refill it now
+
+        quantize_item<P, GSR, SPLIT, false>(Zs, CBP, ntile, ng, gs, srow, tw0, c_base, g, ScaleTables{}, Xq, sX);
         __syncthreads();   // Z and this strip buffer are free again
     }
 }
@@ -701,6 +825,41 @@ cudaError_t launch_k1(const wfq_plan &plan, const void *x_dev, cudaStream_t stre
 }
 
 template <int M, typename Tin, int GSR, int SPLIT>
+int k1i_resident(size_t smem)
+{
+    return resident_ctas_per_sm(input_transform_int_kernel<M, Tin, GSR, SPLIT>, K1_THREADS, smem, 32);
+}
+
+template <int M, typename Tin, int GSR, int SPLIT>
+cudaError_t k1i_setup()
+{
+    auto kern = input_transform_int_kernel<M, Tin, GSR, SPLIT>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                (int)cudaSharedmemCarveoutMaxShared);
+}
+
+template <int M, typename Tin, int GSR, int SPLIT>
+cudaError_t launch_k1i(const wfq_plan &plan, const void *x_dev, cudaStream_t stream)
+{
+    const bool vec = plan.k1iv.vec16 && plan.k1_choice != 3 && (reinterpret_cast<uintptr_t>(x_dev) & 15u) == 0;
+    const K1Params &prm = vec ? plan.k1iv : plan.k1i;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)prm.grid);
+    cfg.blockDim = dim3(K1_THREADS);
+    cfg.dynamicSmemBytes = prm.smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, input_transform_int_kernel<M, Tin, GSR, SPLIT>, static_cast<const Tin *>(x_dev),
+                              plan.ws.Xq, plan.ws.sX, plan.geo, plan.fq, prm);
+}
+
+template <int M, typename Tin, int GSR, int SPLIT>
 int k1n_resident(size_t smem)
 {
     return resident_ctas_per_sm(input_transform_nhwc_kernel<M, Tin, GSR, SPLIT>, K1_THREADS, smem, 32);
@@ -735,7 +894,7 @@ cudaError_t launch_k1n(const wfq_plan &plan, cudaStream_t stream)
 }
 
 // What to do with the instantiation that serves (m, dtype, group size).
-enum K1Op { kK1Launch, kK1Resident, kK1Setup, kK1nLaunch, kK1nResident, kK1nSetup };
+enum K1Op { kK1Launch, kK1Resident, kK1Setup, kK1iLaunch, kK1iResident, kK1iSetup, kK1nLaunch, kK1nResident, kK1nSetup };
 
 template <int M, typename Tin>
 long long k1_by_gs(K1Op op, int gs, const wfq_plan *plan, const void *x, cudaStream_t s, size_t smem)
@@ -745,6 +904,9 @@ long long k1_by_gs(K1Op op, int gs, const wfq_plan *plan, const void *x, cudaStr
         case kK1Launch: return (long long)launch_k1<M, Tin, GSR, SPLIT>(*plan, x, s);  \
         case kK1Resident: return k1_resident<M, Tin, GSR, SPLIT>(smem);                \
         case kK1Setup: return (long long)k1_setup<M, Tin, GSR, SPLIT>();               \
+        case kK1iLaunch: return (long long)launch_k1i<M, Tin, GSR, SPLIT>(*plan, x, s); \
+        case kK1iResident: return k1i_resident<M, Tin, GSR, SPLIT>(smem);              \
+        case kK1iSetup: return (long long)k1i_setup<M, Tin, GSR, SPLIT>();             \
         case kK1nLaunch: return (long long)launch_k1n<M, Tin, GSR, SPLIT>(*plan, s);   \
         case kK1nResident: return k1n_resident<M, Tin, GSR, SPLIT>(smem);              \
         default: return (long long)k1n_setup<M, Tin, GSR, SPLIT>();                    \
@@ -771,7 +933,7 @@ long long k1_op(K1Op op, int m, bool f16, int gs, const wfq_plan *plan, const vo
 
 namespace {
 
-void plan_k1(wfq_plan &plan, K1Params &prm, bool vec16)
+void plan_k1(wfq_plan &plan, K1Params &prm, bool vec16, K1Op resident_op)
 {
     const Geometry &g = plan.geo;
     const bool f16 = plan.in_dtype == WFQ_F16;
@@ -810,7 +972,7 @@ void plan_k1(wfq_plan &plan, K1Params &prm, bool vec16)
     prm.NCB = g.C / prm.CB;
     prm.items = g.N * g.TH * prm.NCH * prm.NCB;
     // persistent CTAs: as many as fit on the device at once
-    const int per_sm = (int)k1_op(kK1Resident, M, f16, g.gs, nullptr, nullptr, nullptr, (size_t)prm.smem);
+    const int per_sm = (int)k1_op(resident_op, M, f16, g.gs, nullptr, nullptr, nullptr, (size_t)prm.smem);
     const int resident = per_sm * (plan.sm_count > 0 ? plan.sm_count : 1);
     prm.grid = prm.items < resident ? prm.items : resident;
 }
@@ -859,9 +1021,13 @@ static void plan_k1_nhwc(wfq_plan &plan)
 // multiple of 8) a second one with 16-byte copies, used when x is 16-byte aligned.
 void plan_input_transform(wfq_plan &plan)
 {
-    plan_k1(plan, plan.k1, false);
+    const bool vec16 = plan.in_dtype == WFQ_F16 && plan.geo.W % 8 == 0;
+    plan_k1(plan, plan.k1, false, kK1Resident);
     plan.k1v = plan.k1;
-    if (plan.in_dtype == WFQ_F16 && plan.geo.W % 8 == 0) plan_k1(plan, plan.k1v, true);
+    if (vec16) plan_k1(plan, plan.k1v, true, kK1Resident);
+    plan_k1(plan, plan.k1i, false, kK1iResident);
+    plan.k1iv = plan.k1i;
+    if (vec16) plan_k1(plan, plan.k1iv, true, kK1iResident);
     plan_k1_nhwc(plan);
     plan.tmap_xn_base = nullptr;
     plan.tmap_xn_tc_base = nullptr;
@@ -875,10 +1041,18 @@ cudaError_t setup_input_transform()
             for (int gs : sizes) {
                 cudaError_t e = (cudaError_t)k1_op(kK1Setup, m, f16 != 0, gs, nullptr, nullptr, nullptr, 0);
                 if (e != cudaSuccess) return e;
+                e = (cudaError_t)k1_op(kK1iSetup, m, f16 != 0, gs, nullptr, nullptr, nullptr, 0);
+                if (e != cudaSuccess) return e;
                 e = (cudaError_t)k1_op(kK1nSetup, m, f16 != 0, gs, nullptr, nullptr, nullptr, 0);
                 if (e != cudaSuccess) return e;
             }
     return cudaSuccess;
+}
+
+// The fully quantized input transform (NCHW input, any group size of the plan).
+cudaError_t launch_input_transform_int(const wfq_plan &plan, const void *x_dev, cudaStream_t stream)
+{
+    return (cudaError_t)k1_op(kK1iLaunch, plan.geo.m, plan.in_dtype == WFQ_F16, plan.geo.gs, &plan, x_dev, stream, 0);
 }
 
 cudaError_t launch_input_transform(wfq_plan &plan, const void *x_dev, cudaStream_t stream)

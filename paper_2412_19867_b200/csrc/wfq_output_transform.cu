@@ -6,6 +6,9 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <type_traits>
+
+#include "wfq_int_quant.cuh"
 #include "wfq_internal.h"
 #include "wfq_ptx.cuh"
 
@@ -88,63 +91,27 @@ __device__ __forceinline__ void epilogue(float (&o)[M], float bias, int act)
 // one array per output row u with the tiles side by side exactly as they lie in the image
 // row, and copies them out with consecutive lanes on consecutive 8 bytes (even W) or
 // consecutive floats (odd W).
-template <int M, int STORE, bool EPI>
-__global__ void __launch_bounds__(128, M == 6 ? (EPI ? 6 : 7) : 8)
-output_transform_kernel(const float *__restrict__ Y, float *__restrict__ y, Geometry g,
-                        ScaleTables tab, const float *__restrict__ bias, int act, int out_half)
+constexpr int TT = 128;                           // tiles per CTA of the output transforms
+
+// What one thread per tile of a CTA's TT tiles has computed goes to y: `row_of(u, o)` gives row u of the
+// thread's tile (called once per u), base is the offset of y[img][k][h0][w0].
+template <int M, int STORE>
+struct StoreShared {
+    float out[STORE != 2 ? M * TT * M : 1];       // [u][tile][v]
+    int tile_base[STORE != 2 ? TT : 1];           // offset of the tile's y[.][.][h0][w0]
+    int tile_lim[STORE != 2 ? TT : 1];            // valid rows * 16 + valid columns
+};
+
+template <int M, int STORE, bool EPI, typename RowOf>
+__device__ __forceinline__ void store_tiles(const RowOf &row_of, StoreShared<M, STORE> &sm, bool live, size_t base,
+                                            int h0, int w0, int k, float *__restrict__ y, const Geometry &g,
+                                            const float *__restrict__ bias, int act, int out_half)
 {
     // 16-bit output (epilogue variants only; out_half 1 = fp16, 2 = bf16): y points at 2-byte storage
     // of the same shape
     [[maybe_unused]] uint16_t *yh = reinterpret_cast<uint16_t *>(y);
-    constexpr int NN = M + 2;
-    constexpr int TT = 128;                       // tiles per CTA
-    __shared__ __align__(16) float out_s[STORE != 2 ? M * TT * M : 1];   // [u][tile][v]
-    __shared__ int tile_base[STORE != 2 ? TT : 1];                       // offset of the tile's y[.][.][h0][w0]
-    __shared__ int tile_lim[STORE != 2 ? TT : 1];                        // valid rows * 16 + valid columns
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    const int k = blockIdx.y;
-    ptx::grid_dependency_wait();   // Y comes from the kernel launched before this one
-    const bool live = t < g.T;
-    if (STORE == 2 && !live) return;
-
-    float tmp[M][NN];
-    int h0 = 0, w0 = 0;
-    size_t base = 0;
-    if (live) {
-        const size_t plane = (size_t)g.K * g.Tp;
-        const float *src = Y + (size_t)k * g.Tp + t;
-        float v[NN][NN];
-#pragma unroll
-        for (int i = 0; i < NN; ++i)
-#pragma unroll
-            for (int j = 0; j < NN; ++j) {
-                v[i][j] = __ldg(src);
-                src += plane;
-            }
-#pragma unroll
-        for (int i = 0; i < NN; ++i)
-#pragma unroll
-            for (int j = 0; j < NN; ++j) v[i][j] *= tab.out_scale[i * NN + j];
-
-        // columns: tmp[u][j] = sum_i VA[u][i] v[i][j]
-#pragma unroll
-        for (int j = 0; j < NN; ++j) {
-            float col[NN], o[M];
-#pragma unroll
-            for (int i = 0; i < NN; ++i) col[i] = v[i][j];
-            at_1d<M>(col, o);
-#pragma unroll
-            for (int u = 0; u < M; ++u) tmp[u][j] = o[u];
-        }
-        const int tw = t % g.TW;
-        const int tq = t / g.TW;
-        const int th = tq % g.TH;
-        const int img = tq / g.TH;
-        h0 = th * M;
-        w0 = tw * M;
-        base = (((size_t)img * g.K + k) * g.H + h0) * g.W + w0;
-    }
-
+    float *out_s = sm.out;
+    int *tile_base = sm.tile_base, *tile_lim = sm.tile_lim;
     if constexpr (STORE != 2) {
         const int j = threadIdx.x;
         if (live) {
@@ -152,7 +119,7 @@ output_transform_kernel(const float *__restrict__ Y, float *__restrict__ y, Geom
 #pragma unroll
             for (int u = 0; u < M; ++u) {
                 float o[M];
-                at_1d<M>(tmp[u], o);
+                row_of(u, o);
                 if constexpr (EPI) epilogue<M>(o, bk, act);
                 float2 *dst = reinterpret_cast<float2 *>(out_s + (u * TT + j) * M);
 #pragma unroll
@@ -206,7 +173,7 @@ output_transform_kernel(const float *__restrict__ Y, float *__restrict__ y, Geom
 #pragma unroll
         for (int u = 0; u < M; ++u) {
             float o[M];
-            at_1d<M>(tmp[u], o);
+            row_of(u, o);
             if constexpr (EPI) epilogue<M>(o, bk, act);
             if (h0 + u < g.H) {
                 if (EPI && out_half) {
@@ -230,6 +197,169 @@ output_transform_kernel(const float *__restrict__ Y, float *__restrict__ y, Geom
             rowh += g.W;
         }
     }
+}
+
+template <int M, int STORE, bool EPI>
+__global__ void __launch_bounds__(TT, M == 6 ? (EPI ? 6 : 7) : 8)
+output_transform_kernel(const float *__restrict__ Y, float *__restrict__ y, Geometry g,
+                        ScaleTables tab, const float *__restrict__ bias, int act, int out_half)
+{
+    constexpr int NN = M + 2;
+    __shared__ __align__(16) StoreShared<M, STORE> sm;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int k = blockIdx.y;
+    ptx::grid_dependency_wait();   // Y comes from the kernel launched before this one
+    const bool live = t < g.T;
+    if (STORE == 2 && !live) return;
+
+    float tmp[M][NN];
+    int h0 = 0, w0 = 0;
+    size_t base = 0;
+    if (live) {
+        const size_t plane = (size_t)g.K * g.Tp;
+        const float *src = Y + (size_t)k * g.Tp + t;
+        float v[NN][NN];
+#pragma unroll
+        for (int i = 0; i < NN; ++i)
+#pragma unroll
+            for (int j = 0; j < NN; ++j) {
+                v[i][j] = __ldg(src);
+                src += plane;
+            }
+#pragma unroll
+        for (int i = 0; i < NN; ++i)
+#pragma unroll
+            for (int j = 0; j < NN; ++j) v[i][j] *= tab.out_scale[i * NN + j];
+
+        // columns: tmp[u][j] = sum_i VA[u][i] v[i][j]
+#pragma unroll
+        for (int j = 0; j < NN; ++j) {
+            float col[NN], o[M];
+#pragma unroll
+            for (int i = 0; i < NN; ++i) col[i] = v[i][j];
+            at_1d<M>(col, o);
+#pragma unroll
+            for (int u = 0; u < M; ++u) tmp[u][j] = o[u];
+        }
+        const int tw = t % g.TW;
+        const int tq = t / g.TW;
+        const int th = tq % g.TH;
+        const int img = tq / g.TH;
+        h0 = th * M;
+        w0 = tw * M;
+        base = (((size_t)img * g.K + k) * g.H + h0) * g.W + w0;
+    }
+
+    auto row_of = [&](int u, float (&o)[M]) { at_1d<M>(tmp[u], o); };
+    store_tiles<M, STORE, EPI>(row_of, sm, live, base, h0, w0, k, y, g, bias, act, out_half);
+}
+
+// ---- the fully quantized output transform (Eq. quant-y) ------------------------------------
+//   y~ = s_qA^2 s_qY  Q(V_A S_A / s_qA)  Q(Y~ / s_qY) Q(S_A V_A^T / s_qA)
+// one thread per (tile, output channel) as above, on integer codes; the results leave through the
+// same stores.
+// MODE 1: one scale per tile; MODE 2: one scale per row, then one per column.
+template <int M, int STORE, int MODE>
+__global__ void __launch_bounds__(TT)
+output_transform_int_kernel(const float *__restrict__ Y, float *__restrict__ y, Geometry g,
+                            const __grid_constant__ FullQuantTables tab, const float *__restrict__ bias, int act, int out_half)
+{
+    constexpr int NN = M + 2;
+    __shared__ __align__(16) StoreShared<M, STORE> sm;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int k = blockIdx.y;
+    ptx::grid_dependency_wait();   // Y comes from the kernel launched before this one
+    const bool live = t < g.T;
+    if (STORE == 2 && !live) return;
+    const size_t plane = (size_t)g.K * g.Tp;
+    const float *src = Y + (size_t)k * g.Tp + (live ? t : 0);
+    float v[NN][NN];
+#pragma unroll
+    for (int i = 0; i < NN; ++i)
+#pragma unroll
+        for (int j = 0; j < NN; ++j) v[i][j] = src[(size_t)(i * NN + j) * plane];
+
+    float out[M][M];
+    if constexpr (MODE == 1) {
+        float amax = 0.f;
+#pragma unroll
+        for (int i = 0; i < NN; ++i)
+#pragma unroll
+            for (int j = 0; j < NN; ++j) amax = fmaxf(amax, fabsf(v[i][j]));
+        const double sqY = __ddiv_rn((double)amax, kIntQmax);
+        const float rinv = __fdiv_rn(127.f, amax);
+        int tmp[NN][M];         // Q(Y) Q(S_A V_A^T): [i][v]
+#pragma unroll
+        for (int i = 0; i < NN; ++i) {
+            int q[NN];
+#pragma unroll
+            for (int j = 0; j < NN; ++j) q[j] = code_of_float(v[i][j], amax, rinv);
+#pragma unroll
+            for (int c = 0; c < M; ++c) {
+                int s = 0;
+#pragma unroll
+                for (int j = 0; j < NN; ++j) s += q[j] * tab.ATq[c * NN + j];
+                tmp[i][c] = s;
+            }
+        }
+        const double sA2 = __dmul_rn(tab.sqA, tab.sqA);
+#pragma unroll
+        for (int u = 0; u < M; ++u)
+#pragma unroll
+            for (int c = 0; c < M; ++c) {
+                int s = 0;
+#pragma unroll
+                for (int i = 0; i < NN; ++i) s += tab.ATq[u * NN + i] * tmp[i][c];
+                out[u][c] = (float)__dmul_rn(__dmul_rn((double)s, sA2), sqY);
+            }
+    } else {
+        double Z[NN][M];        // rows keep their scale: Q(Y_i) Q(S_A V_A^T) s_qA s_row(i)
+#pragma unroll
+        for (int i = 0; i < NN; ++i) {
+            float amax = 0.f;
+#pragma unroll
+            for (int j = 0; j < NN; ++j) amax = fmaxf(amax, fabsf(v[i][j]));
+            const double sr = __ddiv_rn((double)amax, kIntQmax);
+            const float rinv = __fdiv_rn(127.f, amax);
+            int q[NN];
+#pragma unroll
+            for (int j = 0; j < NN; ++j) q[j] = code_of_float(v[i][j], amax, rinv);
+#pragma unroll
+            for (int c = 0; c < M; ++c) {
+                int s = 0;
+#pragma unroll
+                for (int j = 0; j < NN; ++j) s += q[j] * tab.ATq[c * NN + j];
+                Z[i][c] = __dmul_rn(__dmul_rn((double)s, tab.sqA), sr);
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < M; ++c) {
+            double amax = 0.0;
+#pragma unroll
+            for (int i = 0; i < NN; ++i) amax = fmax(amax, fabs(Z[i][c]));
+            const double sc = __ddiv_rn(amax, kIntQmax);
+            const double rc = amax > 0.0 ? __ddiv_rn(1.0, sc) : 0.0;
+            int q[NN];
+#pragma unroll
+            for (int i = 0; i < NN; ++i) q[i] = amax > 0.0 ? code_of(Z[i][c], sc, rc) : 0;
+#pragma unroll
+            for (int u = 0; u < M; ++u) {
+                int s = 0;
+#pragma unroll
+                for (int i = 0; i < NN; ++i) s += tab.ATq[u * NN + i] * q[i];
+                out[u][c] = (float)__dmul_rn(__dmul_rn((double)s, tab.sqA), sc);
+            }
+        }
+    }
+
+    const int tw = t % g.TW, th = (t / g.TW) % g.TH, img = t / (g.TW * g.TH);
+    const int h0 = th * M, w0 = tw * M;
+    const size_t base = (((size_t)img * g.K + k) * g.H + h0) * g.W + w0;
+    auto row_of = [&](int u, float (&o)[M]) {
+#pragma unroll
+        for (int c = 0; c < M; ++c) o[c] = out[u][c];
+    };
+    store_tiles<M, STORE, true>(row_of, sm, live, base, h0, w0, k, y, g, bias, act, out_half);
 }
 
 }  // namespace
@@ -276,31 +406,63 @@ cudaError_t setup_output_transform()
     return e;
 }
 
-cudaError_t launch_output_transform(const wfq_plan &plan, float *y_dev, cudaStream_t stream, bool pdl)
+namespace {
+
+cudaLaunchConfig_t output_config(const wfq_plan &plan, cudaStream_t stream, bool pdl, cudaLaunchAttribute *attr)
 {
-    const Geometry &g = plan.geo;
-    const int threads = 128;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((g.T + threads - 1) / threads, g.K);
-    cfg.blockDim = dim3(threads);
+    cfg.gridDim = dim3((plan.geo.T + TT - 1) / TT, plan.geo.K);
+    cfg.blockDim = dim3(TT);
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr->id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr->val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = pdl ? 1 : 0;
-    // y_dev is 16-byte aligned; rows of an even W keep 8-byte alignment for every tile
-    if (g.m == 2) {
-        if (g.W % 2 == 0) return launch_variant<2, 1>(cfg, plan, y_dev);
-        return launch_variant<2, 0>(cfg, plan, y_dev);
-    }
+    return cfg;
+}
+
+// Calls f with <M, STORE> as integral constants.  y is 16-byte aligned; rows of an even W keep 8-byte
+// alignment for every tile.
+template <typename F>
+cudaError_t with_store(const Geometry &g, F f)
+{
+    using std::integral_constant;
+    if (g.m == 2)
+        return g.W % 2 == 0 ? f(integral_constant<int, 2>{}, integral_constant<int, 1>{})
+                            : f(integral_constant<int, 2>{}, integral_constant<int, 0>{});
     if (g.m == 4) {
-        if (g.W % 4 == 0) return launch_variant<4, 2>(cfg, plan, y_dev);
-        if (g.W % 2 == 0) return launch_variant<4, 1>(cfg, plan, y_dev);
-        return launch_variant<4, 0>(cfg, plan, y_dev);
+        if (g.W % 4 == 0) return f(integral_constant<int, 4>{}, integral_constant<int, 2>{});
+        return g.W % 2 == 0 ? f(integral_constant<int, 4>{}, integral_constant<int, 1>{})
+                            : f(integral_constant<int, 4>{}, integral_constant<int, 0>{});
     }
-    if (g.W % 2 == 0) return launch_variant<6, 1>(cfg, plan, y_dev);
-    return launch_variant<6, 0>(cfg, plan, y_dev);
+    return g.W % 2 == 0 ? f(integral_constant<int, 6>{}, integral_constant<int, 1>{})
+                        : f(integral_constant<int, 6>{}, integral_constant<int, 0>{});
+}
+
+}  // namespace
+
+cudaError_t launch_output_transform(const wfq_plan &plan, float *y_dev, cudaStream_t stream, bool pdl)
+{
+    cudaLaunchAttribute attr[1];
+    const cudaLaunchConfig_t cfg = output_config(plan, stream, pdl, attr);
+    return with_store(plan.geo, [&](auto m, auto store) {
+        return launch_variant<decltype(m)::value, decltype(store)::value>(cfg, plan, y_dev);
+    });
+}
+
+cudaError_t launch_output_transform_int(const wfq_plan &plan, float *y_dev, cudaStream_t stream, bool pdl)
+{
+    cudaLaunchAttribute attr[1];
+    const cudaLaunchConfig_t cfg = output_config(plan, stream, pdl, attr);
+    return with_store(plan.geo, [&](auto m, auto store) {
+        constexpr int M = decltype(m)::value, STORE = decltype(store)::value;
+        const float *Y = plan.ws.Y;
+        if (plan.fq_output == 1)
+            return cudaLaunchKernelEx(&cfg, output_transform_int_kernel<M, STORE, 1>, Y, y_dev, plan.geo, plan.fq,
+                                      plan.bias, plan.act, plan.out_half);
+        return cudaLaunchKernelEx(&cfg, output_transform_int_kernel<M, STORE, 2>, Y, y_dev, plan.geo, plan.fq,
+                                  plan.bias, plan.act, plan.out_half);
+    });
 }
 
 }  // namespace wfq
