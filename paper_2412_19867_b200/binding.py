@@ -159,7 +159,9 @@ def wfq_prepare_filters(plan, w_dev, sB=None, sG=None, sA=None, stream=0):
 
 
 def wfq_conv_forward(plan, x_dev, y_dev, stream=0):
-    _check(load().wfq_conv_forward(plan, x_dev, y_dev, stream), "wfq_conv_forward")
+    status = (_lib or load()).wfq_conv_forward(plan, x_dev, y_dev, stream)
+    if status != WFQ_OK:
+        _check(status, "wfq_conv_forward")
 
 
 def wfq_conv_forward_host(plan, x_host, y_host, stream=0):
@@ -259,6 +261,7 @@ class Conv:
         self.m, self.gs = m, group_size
         self.device = torch.device(device)
         self.in_dtype = in_dtype
+        self.in_layout, self.out_dtype = "nchw", "f32"
         self.plan = wfq_plan_create(N, C, K, H, W, m, 3, group_size, 8)
         wfq_plan_set_input_dtype(self.plan, WFQ_F16 if in_dtype == "f16" else WFQ_F32)
         nbytes = wfq_plan_workspace_bytes(self.plan)
@@ -307,17 +310,24 @@ class Conv:
         wfq_plan_set_epilogue(self.plan, None if bias is None else bias.data_ptr(), act)
 
     def forward(self, x, y=None):
+        # a small layer's kernels take less than this call: nothing here that is not needed per call
         torch = self.torch
         N, C, K, H, W = self.shape
-        xs = (N, H, W, C) if getattr(self, "in_layout", "nchw") == "nhwc" else (N, C, H, W)
-        assert x.is_cuda and x.is_contiguous() and tuple(x.shape) == xs
-        assert x.dtype == (torch.float16 if self.in_dtype == "f16" else torch.float32)
-        ydt = {"f32": torch.float32, "f16": torch.float16, "bf16": torch.bfloat16}[getattr(self, "out_dtype", "f32")]
+        assert x.shape == ((N, H, W, C) if self.in_layout == "nhwc" else (N, C, H, W))
+        assert x.is_cuda and x.is_contiguous()
+        assert x.dtype is (torch.float16 if self.in_dtype == "f16" else torch.float32)
+        out = self.out_dtype
+        ydt = torch.float32 if out == "f32" else torch.float16 if out == "f16" else torch.bfloat16
         if y is None:
             y = torch.empty((N, K, H, W), dtype=ydt, device=self.device)
-        assert y.dtype == ydt and y.is_contiguous() and tuple(y.shape) == (N, K, H, W)
-        with torch.cuda.device(self.device):
-            wfq_conv_forward(self.plan, x.data_ptr(), y.data_ptr(), self._stream())
+        else:
+            assert y.dtype is ydt and y.is_contiguous() and y.shape == (N, K, H, W)
+        here, index = torch.cuda.current_device(), self.device.index
+        if index is None or index == here:
+            wfq_conv_forward(self.plan, x.data_ptr(), y.data_ptr(), torch._C._cuda_getCurrentRawStream(here))
+        else:
+            with torch.cuda.device(self.device):
+                wfq_conv_forward(self.plan, x.data_ptr(), y.data_ptr(), self._stream())
         return y
 
     def forward_host(self, x_host, y_host):
