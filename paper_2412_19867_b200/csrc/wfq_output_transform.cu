@@ -91,19 +91,17 @@ __device__ __forceinline__ void epilogue(float (&o)[M], float bias, int act)
 // one array per output row u with the tiles side by side exactly as they lie in the image
 // row, and copies them out with consecutive lanes on consecutive 8 bytes (even W) or
 // consecutive floats (odd W).
-constexpr int TT = 128;                           // tiles per CTA of the output transforms
-
-// What one thread per tile of a CTA's TT tiles has computed goes to y: `row_of(u, o)` gives row u of the
+// What one thread per tile of a CTA's TT (64 or 128) tiles has computed goes to y: `row_of(u, o)` gives row u of the
 // thread's tile (called once per u), base is the offset of y[img][k][h0][w0].
-template <int M, int STORE>
+template <int M, int STORE, int TT>
 struct StoreShared {
     float out[STORE != 2 ? M * TT * M : 1];       // [u][tile][v]
     int tile_base[STORE != 2 ? TT : 1];           // offset of the tile's y[.][.][h0][w0]
     int tile_lim[STORE != 2 ? TT : 1];            // valid rows * 16 + valid columns
 };
 
-template <int M, int STORE, bool EPI, typename RowOf>
-__device__ __forceinline__ void store_tiles(const RowOf &row_of, StoreShared<M, STORE> &sm, bool live, size_t base,
+template <int M, int STORE, bool EPI, int TT, typename RowOf>
+__device__ __forceinline__ void store_tiles(const RowOf &row_of, StoreShared<M, STORE, TT> &sm, bool live, size_t base,
                                             int h0, int w0, int k, float *__restrict__ y, const Geometry &g,
                                             const float *__restrict__ bias, int act, int out_half)
 {
@@ -199,13 +197,13 @@ __device__ __forceinline__ void store_tiles(const RowOf &row_of, StoreShared<M, 
     }
 }
 
-template <int M, int STORE, bool EPI>
-__global__ void __launch_bounds__(TT, M == 6 ? (EPI ? 6 : 7) : 8)
+template <int M, int STORE, bool EPI, int TT>
+__global__ void __launch_bounds__(TT, (M == 6 ? (EPI ? 6 : 7) : 8) * 128 / TT)
 output_transform_kernel(const float *__restrict__ Y, float *__restrict__ y, Geometry g,
                         ScaleTables tab, const float *__restrict__ bias, int act, int out_half)
 {
     constexpr int NN = M + 2;
-    __shared__ __align__(16) StoreShared<M, STORE> sm;
+    __shared__ __align__(16) StoreShared<M, STORE, TT> sm;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int k = blockIdx.y;
     ptx::grid_dependency_wait();   // Y comes from the kernel launched before this one
@@ -251,7 +249,7 @@ output_transform_kernel(const float *__restrict__ Y, float *__restrict__ y, Geom
     }
 
     auto row_of = [&](int u, float (&o)[M]) { at_1d<M>(tmp[u], o); };
-    store_tiles<M, STORE, EPI>(row_of, sm, live, base, h0, w0, k, y, g, bias, act, out_half);
+    store_tiles<M, STORE, EPI, TT>(row_of, sm, live, base, h0, w0, k, y, g, bias, act, out_half);
 }
 
 // ---- the fully quantized output transform (Eq. quant-y) ------------------------------------
@@ -259,13 +257,13 @@ output_transform_kernel(const float *__restrict__ Y, float *__restrict__ y, Geom
 // one thread per (tile, output channel) as above, on integer codes; the results leave through the
 // same stores.
 // MODE 1: one scale per tile; MODE 2: one scale per row, then one per column.
-template <int M, int STORE, int MODE>
+template <int M, int STORE, int MODE, int TT>
 __global__ void __launch_bounds__(TT)
 output_transform_int_kernel(const float *__restrict__ Y, float *__restrict__ y, Geometry g,
                             const __grid_constant__ FullQuantTables tab, const float *__restrict__ bias, int act, int out_half)
 {
     constexpr int NN = M + 2;
-    __shared__ __align__(16) StoreShared<M, STORE> sm;
+    __shared__ __align__(16) StoreShared<M, STORE, TT> sm;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int k = blockIdx.y;
     ptx::grid_dependency_wait();   // Y comes from the kernel launched before this one
@@ -359,60 +357,58 @@ output_transform_int_kernel(const float *__restrict__ Y, float *__restrict__ y, 
 #pragma unroll
         for (int c = 0; c < M; ++c) o[c] = out[u][c];
     };
-    store_tiles<M, STORE, true>(row_of, sm, live, base, h0, w0, k, y, g, bias, act, out_half);
+    store_tiles<M, STORE, true, TT>(row_of, sm, live, base, h0, w0, k, y, g, bias, act, out_half);
 }
 
 }  // namespace
 
 namespace {
 
-template <int M, int STORE, bool EPI>
-cudaError_t carveout()
+// F(6,3): CTAs of 64 tiles where they leave at least a twentieth fewer threads without a tile than CTAs
+// of 128: 36 tiles of 1280 channels (forward 47.6 -> 45.7 us; of 640 with an epilogue 45.0 -> 38.7 us), 800
+// tiles of 128 channels with an epilogue (36.4 -> 33.7 us), 162 of 256 (26.6 -> 25.9 us).  With about
+// the same number of threads they are no better (121 tiles of 640 channels 41.2 -> 41.8 us, 3200 and 1600
+// tiles within 0.3 us), and F(4,3) and F(2,3) gain nothing from them (32 tiles of 1280 channels 26.5 ->
+// 26.8 us, 3136 tiles of 128 channels 23.9 -> 24.4 us).
+bool half_ctas(const Geometry &g)
 {
-    return cudaFuncSetAttribute(output_transform_kernel<M, STORE, EPI>,
-                                cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+    const long long by64 = ((long long)g.T + 63) / 64 * 64, by128 = ((long long)g.T + 127) / 128 * 128;
+    return g.m == 6 && 20 * by64 <= 19 * by128;
 }
 
-template <int M, int STORE>
-cudaError_t launch_variant(const cudaLaunchConfig_t &cfg, const wfq_plan &plan, float *y_dev)
+// Calls f with <M, STORE, TT> as integral constants.  y is 16-byte aligned; rows of an even W keep 8-byte
+// alignment for every tile.
+template <typename F>
+cudaError_t with_store(int m, int W, bool half, F f)
 {
-    const float *Y = plan.ws.Y;
-    const int out_half = plan.out_half;
-    if (plan.bias || plan.act || out_half)
-        return cudaLaunchKernelEx(&cfg, output_transform_kernel<M, STORE, true>, Y, y_dev, plan.geo, plan.tables,
-                                  plan.bias, plan.act, out_half);
-    return cudaLaunchKernelEx(&cfg, output_transform_kernel<M, STORE, false>, Y, y_dev, plan.geo, plan.tables,
-                              plan.bias, plan.act, out_half);
+    using std::integral_constant;
+    constexpr integral_constant<int, 0> odd{};
+    constexpr integral_constant<int, 1> even{};
+    constexpr integral_constant<int, 2> fours{};
+    constexpr integral_constant<int, 64> t64{};
+    constexpr integral_constant<int, 128> t128{};
+    if (m == 2) {
+        constexpr integral_constant<int, 2> m2{};
+        return W % 2 == 0 ? f(m2, even, t128) : f(m2, odd, t128);
+    }
+    if (m == 4) {
+        constexpr integral_constant<int, 4> m4{};
+        return W % 4 == 0 ? f(m4, fours, t128) : W % 2 == 0 ? f(m4, even, t128) : f(m4, odd, t128);
+    }
+    constexpr integral_constant<int, 6> m6{};
+    if (half) return W % 2 == 0 ? f(m6, even, t64) : f(m6, odd, t64);
+    return W % 2 == 0 ? f(m6, even, t128) : f(m6, odd, t128);
 }
 
-}  // namespace
-
-// One-time attribute setting (per device): the staged variants want six or more CTAs of
-// 10-19 KB of shared memory per SM.
-cudaError_t setup_output_transform()
-{
-    cudaError_t e = carveout<2, 1, false>();
-    if (e == cudaSuccess) e = carveout<2, 0, false>();
-    if (e == cudaSuccess) e = carveout<2, 1, true>();
-    if (e == cudaSuccess) e = carveout<2, 0, true>();
-    if (e == cudaSuccess) e = carveout<4, 1, false>();
-    if (e == cudaSuccess) e = carveout<6, 1, false>();
-    if (e == cudaSuccess) e = carveout<4, 0, false>();
-    if (e == cudaSuccess) e = carveout<6, 0, false>();
-    if (e == cudaSuccess) e = carveout<4, 1, true>();
-    if (e == cudaSuccess) e = carveout<6, 1, true>();
-    if (e == cudaSuccess) e = carveout<4, 0, true>();
-    if (e == cudaSuccess) e = carveout<6, 0, true>();
-    return e;
-}
-
-namespace {
+template <typename F>
+cudaError_t with_store(const Geometry &g, F f) { return with_store(g.m, g.W, half_ctas(g), f); }
 
 cudaLaunchConfig_t output_config(const wfq_plan &plan, cudaStream_t stream, bool pdl, cudaLaunchAttribute *attr)
 {
+    const int tt = half_ctas(plan.geo) ? 64 : 128;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((plan.geo.T + TT - 1) / TT, plan.geo.K);
-    cfg.blockDim = dim3(TT);
+    cfg.gridDim = dim3((plan.geo.T + tt - 1) / tt, plan.geo.K);
+    cfg.blockDim = dim3(tt);
     cfg.stream = stream;
     attr->id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr->val.programmaticStreamSerializationAllowed = 1;
@@ -421,32 +417,41 @@ cudaLaunchConfig_t output_config(const wfq_plan &plan, cudaStream_t stream, bool
     return cfg;
 }
 
-// Calls f with <M, STORE> as integral constants.  y is 16-byte aligned; rows of an even W keep 8-byte
-// alignment for every tile.
-template <typename F>
-cudaError_t with_store(const Geometry &g, F f)
-{
-    using std::integral_constant;
-    if (g.m == 2)
-        return g.W % 2 == 0 ? f(integral_constant<int, 2>{}, integral_constant<int, 1>{})
-                            : f(integral_constant<int, 2>{}, integral_constant<int, 0>{});
-    if (g.m == 4) {
-        if (g.W % 4 == 0) return f(integral_constant<int, 4>{}, integral_constant<int, 2>{});
-        return g.W % 2 == 0 ? f(integral_constant<int, 4>{}, integral_constant<int, 1>{})
-                            : f(integral_constant<int, 4>{}, integral_constant<int, 0>{});
-    }
-    return g.W % 2 == 0 ? f(integral_constant<int, 6>{}, integral_constant<int, 1>{})
-                        : f(integral_constant<int, 6>{}, integral_constant<int, 0>{});
-}
-
 }  // namespace
+
+// One-time attribute setting (per device): the staged variants want twelve or more half CTAs of
+// 5-10 KB of shared memory per SM.
+cudaError_t setup_output_transform()
+{
+    auto carveout = [](auto m, auto store, auto tt) {
+        constexpr int M = decltype(m)::value, STORE = decltype(store)::value, TT = decltype(tt)::value;
+        if (STORE == 2) return cudaSuccess;
+        cudaError_t e = cudaSuccess;
+        for (auto kern : {output_transform_kernel<M, STORE, false, TT>, output_transform_kernel<M, STORE, true, TT>})
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                         (int)cudaSharedmemCarveoutMaxShared);
+        return e;
+    };
+    for (int m = 2; m <= 6; m += 2)
+        for (int W : {1, 2})
+            for (bool half : {false, true}) {
+                const cudaError_t e = with_store(m, W, half, carveout);
+                if (e != cudaSuccess) return e;
+            }
+    return cudaSuccess;
+}
 
 cudaError_t launch_output_transform(const wfq_plan &plan, float *y_dev, cudaStream_t stream, bool pdl)
 {
     cudaLaunchAttribute attr[1];
     const cudaLaunchConfig_t cfg = output_config(plan, stream, pdl, attr);
-    return with_store(plan.geo, [&](auto m, auto store) {
-        return launch_variant<decltype(m)::value, decltype(store)::value>(cfg, plan, y_dev);
+    return with_store(plan.geo, [&](auto m, auto store, auto tt) {
+        constexpr int M = decltype(m)::value, STORE = decltype(store)::value, TT = decltype(tt)::value;
+        const bool epi = plan.bias || plan.act || plan.out_half;
+        return cudaLaunchKernelEx(&cfg, epi ? output_transform_kernel<M, STORE, true, TT>
+                                            : output_transform_kernel<M, STORE, false, TT>,
+                                  (const float *)plan.ws.Y, y_dev, plan.geo, plan.tables, plan.bias, plan.act, plan.out_half);
     });
 }
 
@@ -454,14 +459,11 @@ cudaError_t launch_output_transform_int(const wfq_plan &plan, float *y_dev, cuda
 {
     cudaLaunchAttribute attr[1];
     const cudaLaunchConfig_t cfg = output_config(plan, stream, pdl, attr);
-    return with_store(plan.geo, [&](auto m, auto store) {
-        constexpr int M = decltype(m)::value, STORE = decltype(store)::value;
-        const float *Y = plan.ws.Y;
-        if (plan.fq_output == 1)
-            return cudaLaunchKernelEx(&cfg, output_transform_int_kernel<M, STORE, 1>, Y, y_dev, plan.geo, plan.fq,
-                                      plan.bias, plan.act, plan.out_half);
-        return cudaLaunchKernelEx(&cfg, output_transform_int_kernel<M, STORE, 2>, Y, y_dev, plan.geo, plan.fq,
-                                  plan.bias, plan.act, plan.out_half);
+    return with_store(plan.geo, [&](auto m, auto store, auto tt) {
+        constexpr int M = decltype(m)::value, STORE = decltype(store)::value, TT = decltype(tt)::value;
+        return cudaLaunchKernelEx(&cfg, plan.fq_output == 1 ? output_transform_int_kernel<M, STORE, 1, TT>
+                                                            : output_transform_int_kernel<M, STORE, 2, TT>,
+                                  (const float *)plan.ws.Y, y_dev, plan.geo, plan.fq, plan.bias, plan.act, plan.out_half);
     });
 }
 
