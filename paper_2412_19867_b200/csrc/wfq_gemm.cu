@@ -480,12 +480,24 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                                                   acc[4 * j8 + 1].y, acc[4 * j8 + 2].x, acc[4 * j8 + 2].y,
                                                   acc[4 * j8 + 3].x, acc[4 * j8 + 3].y);
                     } else {
-                        // row = tile: lanes write consecutive t of one Y[p][k][:] row
+                        // row = tile: lanes write consecutive t of one Y[p][k][:] row.  Whole blocks without
+                        // a test per column, the address advanced by the row pitch (forward, 1024 tiles x 320
+                        // channels 44.9 -> 44.2 us, 1600 x 128 44.0 -> 43.0 us; a test per eight columns
+                        // instead costs registers and is slower than a test per column)
                         float *dst = a.Y + ((size_t)p * g.K + col0) * g.Tp + row;
+                        if (col0 + CW <= a.cols) {
 #pragma unroll
-                        for (int j = 0; j < CW / 2; ++j) {
-                            if (col0 + 2 * j < a.cols) dst[(size_t)(2 * j) * g.Tp] = acc[j].x;
-                            if (col0 + 2 * j + 1 < a.cols) dst[(size_t)(2 * j + 1) * g.Tp] = acc[j].y;
+                            for (int j = 0; j < CW / 2; ++j) {
+                                dst[0] = acc[j].x;
+                                dst[g.Tp] = acc[j].y;
+                                dst += 2 * g.Tp;
+                            }
+                        } else {
+#pragma unroll
+                            for (int j = 0; j < CW / 2; ++j) {
+                                if (col0 + 2 * j < a.cols) dst[(size_t)(2 * j) * g.Tp] = acc[j].x;
+                                if (col0 + 2 * j + 1 < a.cols) dst[(size_t)(2 * j + 1) * g.Tp] = acc[j].y;
+                            }
                         }
                     }
                 }
