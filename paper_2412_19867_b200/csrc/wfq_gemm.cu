@@ -202,7 +202,9 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     // Everything above may overlap the kernel that produces Xq and sX.  So may the filter
     // stream, which does not depend on it: before waiting for that kernel the producer loads
     // the filter half of its first stages and asks for the filter tiles of its first units
-    // to be brought into L2 (bounded by a per-CTA share of `l2_prefetch_bytes`).
+    // to be brought into L2 (bounded by a per-CTA share of `l2_prefetch_bytes`).  Filters written by a
+    // kernel before that one are complete: the input transforms let this grid start only after their own
+    // wait for it.
     constexpr int W_ROWS = SWAP ? BM : BN;                 // filter rows of a stage
     // stages of the first unit whose filter half is loaded early
     const int pre = (a.l2_prefetch_bytes > 0 && (int)blockIdx.x < units) ? (KB < NSTAGES ? KB : NSTAGES) : 0;

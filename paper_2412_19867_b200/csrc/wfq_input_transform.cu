@@ -476,14 +476,16 @@ input_transform_kernel(const Tin *__restrict__ x, int8_t *__restrict__ Xq,
     constexpr int NN = M + 2;
     constexpr int P = NN * NN;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    // The contraction kernel launched behind this one may start its prologue and its filter
-    // stream now (it waits for this grid's completion before it touches Xq or sX).
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    // This kernel itself is launched with programmatic stream serialization: it may become
+    // This kernel is launched with programmatic stream serialization: it may become
     // resident while the kernel before it in the stream (normally the previous layer's output
     // transform) drains, and waits here, before its first global access, until that kernel has
     // completed and its writes are visible.
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    ptx::grid_dependency_wait();
+    // The contraction kernel launched behind this one may start its prologue and its filter
+    // stream now (it waits for this grid's completion before it touches Xq or sX).  Not before the
+    // wait: the kernel in front of this one may be the filter preparation, whose codes that stream
+    // reads.  The order costs nothing (forward, 27 layers: 0.1 % less time this way round).
+    ptx::grid_launch_dependents();
     // two strip buffers (the next item is staged while this one is transformed), then Z
     float *Zs = reinterpret_cast<float *>(smem_raw + (1 + prm.dbuf) * prm.strip_bytes);   // [tile][position][CBP]
     const int CBP = prm.CB + 4;   // 16-byte aligned rows an odd number of 16-byte units apart
@@ -571,8 +573,8 @@ input_transform_int_kernel(const Tin *__restrict__ x, int8_t *__restrict__ Xq, f
     constexpr int P = NN * NN;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ float amax_s[(K1_WP - 3) / M][8];               // [tile][run of 32 channels]
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    ptx::grid_dependency_wait();
+    ptx::grid_launch_dependents();
     float *Zs = reinterpret_cast<float *>(smem_raw + (1 + prm.dbuf) * prm.strip_bytes);   // [tile][position][CBP]
     const int CBP = prm.CB + 4;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -700,8 +702,8 @@ input_transform_nhwc_kernel(const __grid_constant__ CUtensorMap tmx, int8_t *__r
     // ends, so the strips start at the next multiple of 128 (the launch adds 128 bytes for this)
     unsigned char *smem_raw = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<uintptr_t>(smem_dyn) + 127) & ~(uintptr_t)127);
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    ptx::grid_dependency_wait();
+    ptx::grid_launch_dependents();
     float *Zs = reinterpret_cast<float *>(smem_raw + (1 + prm.dbuf) * prm.strip_bytes);   // [tile][position][CBP]
     const int CBP = prm.CB + 4;
     const int WB = prm.TB * M + 2;                     // columns of the box

@@ -119,7 +119,6 @@ input_transform_tcn_kernel(const __grid_constant__ CUtensorMap tmx, TnArgs a, Ge
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const WaitCtx ctx{&sh.abort, a.status, a.wait_cycles};
 
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (threadIdx.x == 0) {
         for (int s = 0; s < TN_NSTRIP; ++s) {
             ptx::mbar_init(ptx::smem_u32(&sh.strip_full[s]), 1);
@@ -138,7 +137,7 @@ input_transform_tcn_kernel(const __grid_constant__ CUtensorMap tmx, TnArgs a, Ge
     if (warp == 0) {
         // the producer needs neither the A operand nor TMEM: its first boxes are in flight while the
         // other warps set those up
-        asm volatile("griddepcontrol.wait;" ::: "memory");
+        ptx::grid_dependency_wait();
     } else {
         if (warp == 1) {
             ptx::tmem_alloc(ptx::smem_u32(&sh.tmem_base), C::TMEM_COLS);
@@ -156,7 +155,8 @@ input_transform_tcn_kernel(const __grid_constant__ CUtensorMap tmx, TnArgs a, Ge
         asm volatile("bar.sync 1, %0;" ::"n"(TN_THREADS - 32) : "memory");      // warps 1 ..: operand and TMEM ready
         ptx::tc_fence_after();
         tmem_base = sh.tmem_base;
-        asm volatile("griddepcontrol.wait;" ::: "memory");
+        ptx::grid_dependency_wait();
+        ptx::grid_launch_dependents();      // the contraction's prologue and filter stream may start
     }
 
     const int stride = (int)gridDim.x;

@@ -142,7 +142,10 @@ __device__ __forceinline__ void grid_dependency_wait()
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 // Lets the next grid in the stream start its prologue once every CTA of this grid has
-// got here or exited.
+// got here or exited.  The next grid's prologue may read what grids before this one wrote (the
+// contraction streams filters that filter preparation may just have written), and only this grid's own
+// dependency wait orders it behind those: a grid launched with programmatic serialization calls this
+// after its wait, never before.
 __device__ __forceinline__ void grid_launch_dependents()
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
