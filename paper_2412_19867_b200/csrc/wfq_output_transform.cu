@@ -197,12 +197,17 @@ __device__ __forceinline__ void store_tiles(const RowOf &row_of, StoreShared<M, 
     }
 }
 
-template <int M, int STORE, bool EPI, int TT>
+// LOAD: how Y is loaded, 0 plain, 1 marked for early eviction from L2 (evict_early below), 2 as the flag says.
+// flags: output type (0 fp32, 1 fp16, 2 bf16), plus kEarlyFlag.  One argument for both: a further one makes a launch
+// longer (layers of 12.2 us that wait for launches 12.7 us).
+constexpr int kEarlyFlag = 4;
+template <int M, int STORE, bool EPI, int TT, int LOAD>
 __global__ void __launch_bounds__(TT, (M == 6 ? (EPI ? 6 : 7) : 8) * 128 / TT)
 output_transform_kernel(const float *__restrict__ Y, float *__restrict__ y, Geometry g,
-                        ScaleTables tab, const float *__restrict__ bias, int act, int out_half)
+                        ScaleTables tab, const float *__restrict__ bias, int act, int flags)
 {
     constexpr int NN = M + 2;
+    const int out_half = flags & (kEarlyFlag - 1);
     __shared__ __align__(16) StoreShared<M, STORE, TT> sm;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int k = blockIdx.y;
@@ -217,9 +222,6 @@ output_transform_kernel(const float *__restrict__ Y, float *__restrict__ y, Geom
         const size_t plane = (size_t)g.K * g.Tp;
         const float *src = Y + (size_t)k * g.Tp + t;
         float v[NN][NN];
-        // Y is read once.  Marked for early eviction it leaves L2 first, which helps where it is large
-        // (forward, 3200 tiles 44.6 -> 43.4 us, 1024 tiles 46.0 -> 45.0 us) and hurts where it is small (64 tiles
-        // 9.8 -> 10.3 us); small F(6,3) layers gain a little from passing L1 by (36 tiles 39.3 -> 38.3 us).
         auto load = [&](auto one) {
 #pragma unroll
             for (int i = 0; i < NN; ++i)
@@ -229,7 +231,7 @@ output_transform_kernel(const float *__restrict__ Y, float *__restrict__ y, Geom
                     src += plane;
                 }
         };
-        if (TT == 128 && g.T >= 512) load([](const float *q) { return __ldcs(q); });
+        if (LOAD == 1 || (LOAD == 2 && (flags & kEarlyFlag))) load([](const float *q) { return __ldcs(q); });
         else if (M == 6) load([](const float *q) { return __ldcg(q); });
         else load([](const float *q) { return __ldg(q); });
 #pragma unroll
@@ -384,6 +386,33 @@ bool half_ctas(const Geometry &g)
     return g.m == 6 && 20 * by64 <= 19 * by128;
 }
 
+// How Y, which is read once, is loaded.  Marked for early eviction it leaves L2 before what the next kernels
+// read.  That helps where Y takes a good part of the 126 MB of L2 (forward, F(6,3), plain -> marked: 33 MB 28.4 ->
+// 28.1 us, 66 MB 47.5 -> 45.9 us, 98 MB 73.5 -> 69.1 us, 133 MB 92.4 -> 89.1 us; F(4,3) 47 MB 45.3 -> 44.5 us, 94 MB
+// 77.2 -> 73.4 us; F(2,3) 51 MB 39.4 -> 38.5 us) and is no better or worse where it is small (20 MB 22.8 -> 23.0 us,
+// 24 MB 25.3 -> 25.6 us).  With Y and y together beyond twice L2 most of Y has left by itself, and F(6,3) is better
+// off without the mark (Y 199 MB with fp32 y 125.8 -> 127.5 us, 393 MB 227.6 -> 238.8 us; 199 MB with fp16 y, just below
+// the limit, 127.2 -> 124.7 us); F(4,3) and F(2,3) are not (377 MB 131.4 -> 129.0 us, 336 MB 165.2 -> 158.3 us).
+bool evict_early(const wfq_plan &plan)
+{
+    const Geometry &g = plan.geo;
+    const size_t Y = (size_t)g.P * g.K * g.Tp * sizeof(float);
+    const size_t y = (size_t)g.N * g.K * g.H * g.W * (plan.out_half ? 2 : 4);
+    return Y >= (size_t)32 << 20 && (g.m != 6 || Y + y <= (size_t)256 << 20);
+}
+// With two forms of the loads in the kernel the compiler issues all of them before the arithmetic, which is faster
+// than one form scheduled into it (forward, 600 tiles of 320 channels 35.5 -> 34.5 us, 243 of 128 14.2 -> 13.8 us, F(4,3)
+// 2048 of 128 24.3 -> 24.0 us).  The F(6,3) variants with an epilogue have no registers for it (80 with 4 to 16 bytes
+// spilled; 256 tiles of 1280 channels 80.9 us, with one form 75.8 us).
+constexpr bool both_loads(int m, bool epi, int tt) { return tt == 128 && !(m == 6 && epi); }
+
+template <int M, int STORE, bool EPI, int TT>
+auto variant(bool early)
+{
+    if constexpr (both_loads(M, EPI, TT)) return output_transform_kernel<M, STORE, EPI, TT, 2>;
+    else return early ? output_transform_kernel<M, STORE, EPI, TT, 1> : output_transform_kernel<M, STORE, EPI, TT, 0>;
+}
+
 // Calls f with <M, STORE, TT> as integral constants.  y is 16-byte aligned; rows of an even W keep 8-byte
 // alignment for every tile.
 template <typename F>
@@ -435,7 +464,8 @@ cudaError_t setup_output_transform()
         constexpr int M = decltype(m)::value, STORE = decltype(store)::value, TT = decltype(tt)::value;
         if (STORE == 2) return cudaSuccess;
         cudaError_t e = cudaSuccess;
-        for (auto kern : {output_transform_kernel<M, STORE, false, TT>, output_transform_kernel<M, STORE, true, TT>})
+        for (auto kern : {variant<M, STORE, false, TT>(false), variant<M, STORE, false, TT>(true),
+                          variant<M, STORE, true, TT>(false), variant<M, STORE, true, TT>(true)})
             if (e == cudaSuccess)
                 e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
                                          (int)cudaSharedmemCarveoutMaxShared);
@@ -456,10 +486,10 @@ cudaError_t launch_output_transform(const wfq_plan &plan, float *y_dev, cudaStre
     const cudaLaunchConfig_t cfg = output_config(plan, stream, pdl, attr);
     return with_store(plan.geo, [&](auto m, auto store, auto tt) {
         constexpr int M = decltype(m)::value, STORE = decltype(store)::value, TT = decltype(tt)::value;
-        const bool epi = plan.bias || plan.act || plan.out_half;
-        return cudaLaunchKernelEx(&cfg, epi ? output_transform_kernel<M, STORE, true, TT>
-                                            : output_transform_kernel<M, STORE, false, TT>,
-                                  (const float *)plan.ws.Y, y_dev, plan.geo, plan.tables, plan.bias, plan.act, plan.out_half);
+        const bool epi = plan.bias || plan.act || plan.out_half, early = evict_early(plan);
+        return cudaLaunchKernelEx(&cfg, epi ? variant<M, STORE, true, TT>(early) : variant<M, STORE, false, TT>(early),
+                                  (const float *)plan.ws.Y, y_dev, plan.geo, plan.tables, plan.bias, plan.act,
+                                  plan.out_half | (early ? kEarlyFlag : 0));
     });
 }
 
