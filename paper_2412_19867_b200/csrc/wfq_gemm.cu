@@ -483,9 +483,12 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                                                   acc[4 * j8 + 3].x, acc[4 * j8 + 3].y);
                     } else {
                         // row = tile: lanes write consecutive t of one Y[p][k][:] row.  Whole blocks without
-                        // a test per column, the address advanced by the row pitch (forward, 1024 tiles x 320
-                        // channels 44.9 -> 44.2 us, 1600 x 128 44.0 -> 43.0 us; a test per eight columns
-                        // instead costs registers and is slower than a test per column)
+                        // a test per column, the address advanced by the row pitch (forward, F(4,3), 784 tiles x
+                        // 320 channels 34.4 -> 33.6 us, F(6,3), 1600 x 320 78.4 -> 76.8 us).  A last block of
+                        // fewer columns ends at the first group of eight without one, which the tests of every
+                        // column did not (1600 tiles x 8 channels 23.1 -> 21.4 us, x 40 24.9 -> 24.0 us, x 136
+                        // 40.4 -> 39.3 us; with tests alone it was slower than before the whole blocks had
+                        // their own loop, 22.5 us for 8 channels)
                         float *dst = a.Y + ((size_t)p * g.K + col0) * g.Tp + row;
                         if (col0 + CW <= a.cols) {
 #pragma unroll
@@ -497,6 +500,7 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                         } else {
 #pragma unroll
                             for (int j = 0; j < CW / 2; ++j) {
+                                if (j % 4 == 0 && col0 + 2 * j >= a.cols) break;
                                 if (col0 + 2 * j < a.cols) dst[(size_t)(2 * j) * g.Tp] = acc[j].x;
                                 if (col0 + 2 * j + 1 < a.cols) dst[(size_t)(2 * j + 1) * g.Tp] = acc[j].y;
                             }
