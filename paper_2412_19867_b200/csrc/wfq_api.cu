@@ -46,6 +46,18 @@ constexpr int kMaxDevices = 64;
 std::mutex g_setup_mutex;
 bool g_device_ready[kMaxDevices];
 
+// Attributes and launch shapes of the integer input transform for a plan that uses it and knows its device.
+wfq_status_t plan_int_mode(wfq_plan *plan)
+{
+    if (!plan->fq_input || plan->sm_count == 0) return WFQ_OK;
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess) return WFQ_ERR_CUDA;
+    if (dev != plan->device && cudaSetDevice(plan->device) != cudaSuccess) return WFQ_ERR_CUDA;
+    const cudaError_t e = wfq::plan_input_transform_int(*plan);
+    if (dev != plan->device && cudaSetDevice(dev) != cudaSuccess) return WFQ_ERR_CUDA;
+    return cuda_status(e);
+}
+
 wfq_status_t bind_device(wfq_plan *plan)
 {
     int dev = -1;
@@ -71,7 +83,9 @@ wfq_status_t bind_device(wfq_plan *plan)
     plan->sm_count = sms;
     wfq::plan_input_transform(*plan);
     wfq::plan_input_transform_tc(*plan);
-    return WFQ_OK;
+    const wfq_status_t s = plan_int_mode(plan);
+    if (s != WFQ_OK) plan->sm_count = 0;      // not bound: the next call tries again
+    return s;
 }
 
 }  // namespace
@@ -190,7 +204,7 @@ wfq_status_t wfq_plan_set_input_dtype(wfq_plan_t *plan, wfq_dtype_t dtype)
         wfq::plan_input_transform(*plan);
         wfq::plan_input_transform_tc(*plan);
     }
-    return WFQ_OK;
+    return plan_int_mode(plan);
 }
 
 wfq_status_t wfq_plan_set_input_layout(wfq_plan_t *plan, wfq_layout_t layout)
@@ -252,10 +266,18 @@ wfq_status_t wfq_plan_set_full_quant(wfq_plan_t *plan, int quant_input, wfq_y_qu
     if (quant_input != 0 && quant_input != 1) return WFQ_ERR_INVALID_ARG;
     if (y_mode != WFQ_Y_FP32 && y_mode != WFQ_Y_TILE && y_mode != WFQ_Y_ROW) return WFQ_ERR_INVALID_ARG;
     if (quant_input && (plan->geo.gs % 32 != 0 || plan->geo.gs > 256 || plan->in_nhwc)) return WFQ_ERR_UNSUPPORTED;
-    plan->fq_input = quant_input != 0;
-    plan->fq_output = (int)y_mode;
-    for (int i = 0; i < 2; ++i)
-        if (plan->sub[i]) { plan->sub[i]->fq_input = plan->fq_input; plan->sub[i]->fq_output = plan->fq_output; }
+    for (wfq_plan *p : {plan, plan->sub[0], plan->sub[1]}) {
+        if (!p) continue;
+        if (p->fq_input != (quant_input != 0)) {
+            p->fq_input = quant_input != 0;
+            const wfq_status_t s = plan_int_mode(p);
+            if (s != WFQ_OK) {
+                p->fq_input = false;
+                return s;
+            }
+        }
+        p->fq_output = (int)y_mode;
+    }
     return WFQ_OK;
 }
 
@@ -546,7 +568,9 @@ static wfq_status_t setup_host_pipeline(wfq_plan *plan)
             plan->sub[s]->borrowed = true;
         }
         wfq_plan *q = plan->sub[s];
-        wfq_plan_set_input_dtype(q, plan->in_dtype);
+        q->fq_input = plan->fq_input; q->fq_output = plan->fq_output;
+        wfq_status_t st = wfq_plan_set_input_dtype(q, plan->in_dtype);
+        if (st != WFQ_OK) return st;
         q->k1_choice = plan->k1_choice;
         q->in_nhwc = plan->in_nhwc;
         // same orientation of the contraction as the whole batch: identical arithmetic
@@ -554,14 +578,14 @@ static wfq_status_t setup_host_pipeline(wfq_plan *plan)
         q->gemm_bn = plan->gemm_bn;
         const size_t slice = align_up(q->ws.total, 1024);
         if (2 * slice > plan->ws.total) return WFQ_ERR_UNSUPPORTED;
-        wfq_status_t st = wfq_plan_set_workspace(q, reinterpret_cast<char *>(plan->ws.Xq) + s * slice, slice);
+        st = wfq_plan_set_workspace(q, reinterpret_cast<char *>(plan->ws.Xq) + s * slice, slice);
         if (st != WFQ_OK) return st;
         q->Wq = plan->Wq; q->sW = plan->sW; q->status = plan->status;
         q->tables = plan->tables;
         q->tmap_wq = plan->tmap_wq; q->tmap_wq_ok = plan->tmap_wq_ok;
         q->wait_cycles = plan->wait_cycles;
         q->bias = plan->bias; q->act = plan->act; q->out_half = plan->out_half;
-        q->fq_input = plan->fq_input; q->fq_output = plan->fq_output; q->fq = plan->fq;
+        q->fq = plan->fq;
         q->prepared = true;
         if (!plan->host_stream[s] &&
             cudaStreamCreateWithFlags(&plan->host_stream[s], cudaStreamNonBlocking) != cudaSuccess)

@@ -26,16 +26,12 @@
 // the group in registers.
 #include <cuda_fp16.h>
 
-#include "wfq_int_quant.cuh"
 #include "wfq_internal.h"
 #include "wfq_ptx.cuh"
+#include "wfq_strip.cuh"
 
 namespace wfq {
 namespace {
-
-constexpr int K1_THREADS = 128;
-constexpr int K1_WP = 16;        // staged columns per row (image columns w_base .. w_base+15)
-constexpr int K1_WPV = 24;       // the same where rows are copied in aligned 16-byte pieces (w_base a multiple of 8)
 
 // ---- 1-D input transforms with the standard B^T ------------------------------------
 
@@ -132,230 +128,6 @@ __device__ __forceinline__ void bt_1d(const float2 (&d)[8], float2 (&r)[8])
 __device__ __forceinline__ float to_float32(float v) { return v; }
 __device__ __forceinline__ float to_float32(__half v) { return __half2float(v); }
 
-// ---- patch load from the staged strip ---------------------------------------------
-// `ch` points at the channel's plane in smem; `col0` is the (even) smem column whose
-// successor is the tile's first input column.
-template <int NN>
-__device__ __forceinline__ void load_patch(const __half *ch, int col0, float (&d)[NN][NN])
-{
-#pragma unroll
-    for (int a = 0; a < NN; ++a) {
-        const __half2 *row = reinterpret_cast<const __half2 *>(ch + a * K1_WP + col0);
-        float v[NN + 2];
-#pragma unroll
-        for (int w = 0; w < (NN + 2) / 2; ++w) {
-            const float2 f = __half22float2(row[w]);
-            v[2 * w] = f.x;
-            v[2 * w + 1] = f.y;
-        }
-#pragma unroll
-        for (int b = 0; b < NN; ++b) d[a][b] = v[b + 1];
-    }
-}
-
-// The same from a strip staged in 16-byte pieces (rows of K1_WPV columns, channel stride a
-// multiple of 16 bytes and an odd number of 16-byte units): 16-byte loads, for which the eight
-// lanes of a quarter warp then hit eight different groups of four banks.  `k0` is the first of
-// the two 16-byte pieces that hold columns col0 .. col0 + NN + 1, WO the 32-bit word of col0
-// inside them (col0 is even); both are the same for all lanes of the warp.
-template <int NN, int WO>
-__device__ __forceinline__ void load_patch_vec(const __half *ch, int k0, float (&d)[NN][NN])
-{
-#pragma unroll
-    for (int a = 0; a < NN; ++a) {
-        const uint4 *row = reinterpret_cast<const uint4 *>(ch + a * K1_WPV) + k0;
-        const uint4 q0 = row[0], q1 = row[1];
-        const uint32_t w[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
-        float v[NN + 2];
-#pragma unroll
-        for (int i = 0; i < (NN + 2) / 2; ++i) {
-            const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&w[WO + i]));
-            v[2 * i] = f.x;
-            v[2 * i + 1] = f.y;
-        }
-#pragma unroll
-        for (int b = 0; b < NN; ++b) d[a][b] = v[b + 1];
-    }
-}
-template <int NN>
-__device__ __forceinline__ void load_patch_vec(const __half *ch, int col0, float (&d)[NN][NN])
-{
-    const int k0 = col0 >> 3;
-    switch ((col0 & 7) >> 1) {            // warp-uniform
-        case 0: load_patch_vec<NN, 0>(ch, k0, d); break;
-        case 1: load_patch_vec<NN, 1>(ch, k0, d); break;
-        case 2: load_patch_vec<NN, 2>(ch, k0, d); break;
-        default: load_patch_vec<NN, 3>(ch, k0, d); break;
-    }
-}
-template <int NN>
-__device__ __forceinline__ void load_patch_vec(const float *, int, float (&)[NN][NN]) {}   // fp16 only
-
-template <int NN>
-__device__ __forceinline__ void load_patch(const float *ch, int col0, float (&d)[NN][NN])
-{
-#pragma unroll
-    for (int a = 0; a < NN; ++a)
-#pragma unroll
-        for (int b = 0; b < NN; ++b) d[a][b] = ch[a * K1_WP + col0 + 1 + b];
-}
-
-// Codes: round v*inv to the nearest integer (ties to even) and keep the low byte.
-// fl32(v*inv) + 1.5*2^23 is exact up to the rounding to an integer, and the sum's bit
-// pattern is 0x4B400000 + q for |q| <= 2^22.
-// Packed f32x2 multiply (one instruction for two products, each correctly rounded).
-__device__ __forceinline__ float2 mul2_rn(float2 a, float2 b)
-{
-    float2 d;
-    asm("{\n\t.reg .b64 ra, rb, rd;\n\t"
-        "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
-        "mul.rn.f32x2 rd, ra, rb;\n\t"
-        "mov.b64 {%0, %1}, rd;\n\t}"
-        : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-    return d;
-}
-
-// One code: fl32(v*inv), then + 1.5*2^23; two separately rounded scalar operations, as
-// the quantizer is defined.  (A packed multiply followed by a packed add, written as
-// intrinsics or as PTX, came out as one fused multiply-add: it rounds once and decides
-// near-ties differently, and a single differing code of an outlier-dominated group can
-// move the final output by more than the end-to-end tolerance.)
-__device__ __forceinline__ uint32_t code_bits(float v, float inv)
-{
-    return __float_as_uint(__fadd_rn(__fmul_rn(v, inv), 12582912.f));
-}
-__device__ __forceinline__ uint32_t codes4(float4 v, float inv)
-{
-    return __byte_perm(__byte_perm(code_bits(v.x, inv), code_bits(v.y, inv), 0x0040),
-                       __byte_perm(code_bits(v.z, inv), code_bits(v.w, inv), 0x0040), 0x5410);
-}
-
-// X = Z * (s + sl), rounded once: fma(z, s, z * sl) (the factor is held as two floats).
-__device__ __forceinline__ float4 scale4(float4 v, float2 s2, float2 sl2)
-{
-    const float2 a = make_float2(v.x, v.y), b = make_float2(v.z, v.w);
-    const float2 lo = __ffma2_rn(a, s2, mul2_rn(a, sl2));
-    const float2 hi = __ffma2_rn(b, s2, mul2_rn(b, sl2));
-    return make_float4(lo.x, lo.y, hi.x, hi.y);
-}
-
-__device__ __forceinline__ float absmax4(float m, float4 v)
-{
-    return fmaxf(fmaxf(fmaxf(m, fabsf(v.x)), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)));
-}
-
-// 32-byte store (one full sector); `p` must be 32-byte aligned.
-__device__ __forceinline__ void st_global_v8_b32(void *p, uint32_t a, uint32_t b, uint32_t c, uint32_t d,
-                                                 uint32_t e, uint32_t f, uint32_t g, uint32_t h)
-{
-    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
-                 ::"l"(p), "r"(a), "r"(b), "r"(c), "r"(d), "r"(e), "r"(f), "r"(g), "r"(h)
-                 : "memory");
-}
-
-__device__ __forceinline__ void cp_async_4(uint32_t dst, const void *src, bool valid)
-{
-    const int n = valid ? 4 : 0;   // 0 source bytes: the destination is zero filled
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
-}
-__device__ __forceinline__ void cp_async_16(uint32_t dst, const void *src, bool valid)
-{
-    const int n = valid ? 16 : 0;
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit()
-{
-    asm volatile("cp.async.commit_group;" ::: "memory");
-}
-template <int N>
-__device__ __forceinline__ void cp_async_wait_group()   // all but the N newest groups are done
-{
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
-// ---- strip staging -----------------------------------------------------------------
-// smem column j of the strip holds image column w_base + j (w_base even); rows are
-// image rows h_base .. h_base + NN - 1; anything outside the image is zero.
-template <typename Tin, int NN>
-__device__ __forceinline__ void stage_strip(Tin *sm, const Tin *__restrict__ x, const Geometry &g,
-                                            const K1Params &prm, int img, int c_base, int h_base,
-                                            int w_base)
-{
-    const size_t HW = (size_t)g.H * g.W;
-    const Tin *ximg = x + ((size_t)img * g.C + c_base) * HW;
-    // Each thread owns one (row, column) slot of the strip and walks over the channels,
-    // so its bounds test and addresses are computed once.
-    if (sizeof(Tin) == 2 && prm.vec16) {
-        // 16-byte pieces: W and w_base are multiples of 8 and x is 16-byte aligned, so a piece
-        // lies inside the image or outside it as a whole
-        constexpr int CPR = K1_WPV / 8;                        // copies per row
-        constexpr int ROWS = K1_THREADS / CPR;
-        constexpr int CSLOTS = ROWS / NN;
-        const int jc = threadIdx.x % CPR;
-        const int rs = threadIdx.x / CPR;
-        const int a = rs % NN, cslot = rs / NN;
-        if (cslot < CSLOTS) {
-            const int h = h_base + a, w = w_base + 8 * jc;
-            const bool ok = h >= 0 && h < g.H && w >= 0 && w < g.W;
-            const Tin *src = ok ? ximg + (size_t)cslot * HW + (size_t)h * g.W + w : x;
-            const size_t src_step = ok ? (size_t)CSLOTS * HW : 0;
-            uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(sm)) +
-                           (uint32_t)((cslot * prm.CS + a * K1_WPV + 8 * jc) * sizeof(Tin));
-            const uint32_t dst_step = (uint32_t)(CSLOTS * prm.CS * sizeof(Tin));
-            for (int c = cslot; c < prm.CB; c += CSLOTS) {
-                cp_async_16(dst, src, ok);
-                src += src_step;
-                dst += dst_step;
-            }
-        }
-    } else if (sizeof(Tin) == 4 || prm.pair) {
-        constexpr int EPC = sizeof(Tin) == 4 ? 1 : 2;          // elements per 4-byte copy
-        constexpr int CPR = K1_WP / EPC;                       // copies per row
-        constexpr int ROWS = K1_THREADS / CPR;                 // rows covered by one pass
-        constexpr int CSLOTS = ROWS / NN;                      // channels covered by one pass
-        const int jc = threadIdx.x % CPR;
-        const int rs = threadIdx.x / CPR;
-        const int a = rs % NN, cslot = rs / NN;
-        if (cslot < CSLOTS) {
-            const int h = h_base + a, w = w_base + EPC * jc;
-            const bool ok = h >= 0 && h < g.H && w >= 0 && w < g.W;   // W even for pairs: both or none
-            const Tin *src = ok ? ximg + (size_t)cslot * HW + (size_t)h * g.W + w : x;
-            const size_t src_step = ok ? (size_t)CSLOTS * HW : 0;
-            uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(sm)) +
-                           (uint32_t)((cslot * prm.CS + a * K1_WP + EPC * jc) * sizeof(Tin));
-            const uint32_t dst_step = (uint32_t)(CSLOTS * prm.CS * sizeof(Tin));
-            for (int c = cslot; c < prm.CB; c += CSLOTS) {
-                cp_async_4(dst, src, ok);
-                src += src_step;
-                dst += dst_step;
-            }
-        }
-    } else {
-        // fp16 with an odd W or a 2-byte aligned base: plain 2-byte loads, eight channels
-        // in flight per thread (these copies are complete when the function returns)
-        constexpr int ROWS = K1_THREADS / K1_WP;               // 8 row slots per pass
-        constexpr int CSLOTS = ROWS / NN;                      // 1
-        const int j = threadIdx.x % K1_WP;
-        const int rs = threadIdx.x / K1_WP;
-        const int a = rs % NN, cslot = rs / NN;
-        if (cslot < CSLOTS) {
-            const int h = h_base + a, w = w_base + j;
-            const bool ok = h >= 0 && h < g.H && w >= 0 && w < g.W;
-            const Tin *src = ximg + (size_t)cslot * HW + (size_t)h * g.W + w;
-            Tin *dst = sm + cslot * prm.CS + a * K1_WP + j;
-            for (int c = cslot; c < prm.CB; c += 8 * CSLOTS) {     // CB is a multiple of 32
-                Tin v[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) v[u] = ok ? __ldg(src + (size_t)u * CSLOTS * HW) : Tin(0);
-#pragma unroll
-                for (int u = 0; u < 8; ++u) dst[u * CSLOTS * prm.CS] = v[u];
-                src += (size_t)8 * CSLOTS * HW;
-                dst += 8 * CSLOTS * prm.CS;
-            }
-        }
-    }
-}
-
 // Z = B^T d B with the standard B^T, written to out[p * pitch] for p = i*NN + j.
 template <int NN>
 __device__ __forceinline__ void transform_patch(float (&d)[NN][NN], float *__restrict__ out, int pitch)
@@ -378,89 +150,6 @@ __device__ __forceinline__ void transform_patch(float (&d)[NN][NN], float *__res
         bt_1d(d[i], r);
 #pragma unroll
         for (int j = 0; j < NN; ++j) out[(i * NN + j) * pitch] = r[j];
-    }
-}
-
-// ---- group abs-max and scale (the quantizer of Section 2, one scale per group) ------
-// amax >= 0.  Returns the stored scale and the reciprocal used for the codes.
-__device__ __forceinline__ void group_scale(float amax, float &scale, float &inv)
-{
-    const bool nz = amax >= 1e-30f;
-    scale = nz ? __fdiv_rn(amax, 127.f) : 0.f;
-    inv = nz ? __fdiv_rn(127.f, amax) : 0.f;
-}
-
-// ---- phase 2 of a work item: quantize, one (tile, group, position) per thread -------------
-// Zs holds the transformed values of `ntile` tiles as [tile][position][CB + 4] fp32; the item is
-// tiles tw0 .. of tile row `srow` (= image * TH + tile row) and channels c_base .. c_base + CB.
-template <int P, int GSR, int SPLIT, bool SCALED = true>
-__device__ __forceinline__ void quantize_item(const float *__restrict__ Zs, int CBP, int ntile, int ng, int gs,
-                                              int srow, int tw0, int c_base, const Geometry &g,
-                                              const ScaleTables &tab, int8_t *__restrict__ Xq,
-                                              float *__restrict__ sX)
-{
-    // X = Z * (caller's per-position factor) is formed here, one rounding, as the
-    // quantizer's input; then abs-max, scale, reciprocal and codes.
-    const int g_base = c_base / gs;
-    if constexpr (GSR > 0) {
-        // whole warps walk the loop so that the lanes sharing a group can shuffle
-        const int tasks = ntile * ng * P * SPLIT;
-        for (int base = 0; base < tasks; base += K1_THREADS) {
-            const int task = base + (int)threadIdx.x;
-            const bool act = task < tasks;          // the lanes of a group are all in or all out
-            const int tk = act ? task : 0;
-            const int part = tk % SPLIT, rest = tk / SPLIT;
-            const int q = rest / P, p = rest - q * P;
-            const int tl = q / ng, grp = q - tl * ng;
-            const int t = srow * g.TW + tw0 + tl;
-            const float4 *src = reinterpret_cast<const float4 *>(Zs + (size_t)(tl * P + p) * CBP + grp * gs +
-                                                                 part * GSR);
-            int8_t *dst = Xq + ((size_t)p * g.T + t) * g.C + c_base + grp * gs + part * GSR;
-            const float sp = tab.in_scale[p], sl = tab.in_scale_lo[p];
-            const float2 sp2 = make_float2(sp, sp), sl2 = make_float2(sl, sl);
-            float4 v[GSR / 4];
-            float amax = 0.f;
-#pragma unroll
-            for (int k = 0; k < GSR / 4; ++k) {
-                v[k] = SCALED ? scale4(src[k], sp2, sl2) : src[k];
-                amax = absmax4(amax, v[k]);
-            }
-            if constexpr (SPLIT >= 2) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 1));
-            if constexpr (SPLIT >= 4) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 2));
-            float scale, inv;
-            group_scale(amax, scale, inv);
-            if (act) {
-#pragma unroll
-                for (int k = 0; k < GSR / 32; ++k)        // 32 codes = one full sector per store
-                    st_global_v8_b32(dst + 32 * k, codes4(v[8 * k], inv), codes4(v[8 * k + 1], inv),
-                                     codes4(v[8 * k + 2], inv), codes4(v[8 * k + 3], inv),
-                                     codes4(v[8 * k + 4], inv), codes4(v[8 * k + 5], inv),
-                                     codes4(v[8 * k + 6], inv), codes4(v[8 * k + 7], inv));
-                if (part == 0) sX[((size_t)p * g.G + g_base + grp) * g.Ts + t] = scale;
-            }
-        }
-    } else {
-        const int tasks = ntile * ng * P;
-        for (int task = threadIdx.x; task < tasks; task += K1_THREADS) {
-            const int q = task / P, p = task - q * P;
-            const int tl = q / ng, grp = q - tl * ng;
-            const int t = srow * g.TW + tw0 + tl;
-            const float4 *src = reinterpret_cast<const float4 *>(Zs + (size_t)(tl * P + p) * CBP + grp * gs);
-            int8_t *dst = Xq + ((size_t)p * g.T + t) * g.C + c_base + grp * gs;
-            const float sp = tab.in_scale[p], sl = tab.in_scale_lo[p];
-            const float2 sp2 = make_float2(sp, sp), sl2 = make_float2(sl, sl);
-            auto val = [&](int k) { return SCALED ? scale4(src[k], sp2, sl2) : src[k]; };
-            float scale, inv;
-            float amax = 0.f;
-            for (int k = 0; k < gs / 4; ++k) amax = absmax4(amax, val(k));
-            group_scale(amax, scale, inv);
-            for (int k = 0; k < gs / 32; ++k)
-                st_global_v8_b32(dst + 32 * k, codes4(val(8 * k), inv), codes4(val(8 * k + 1), inv),
-                                 codes4(val(8 * k + 2), inv), codes4(val(8 * k + 3), inv),
-                                 codes4(val(8 * k + 4), inv), codes4(val(8 * k + 5), inv),
-                                 codes4(val(8 * k + 6), inv), codes4(val(8 * k + 7), inv));
-            sX[((size_t)p * g.G + g_base + grp) * g.Ts + t] = scale;
-        }
     }
 }
 
@@ -550,128 +239,6 @@ input_transform_kernel(const Tin *__restrict__ x, int8_t *__restrict__ Xq,
         if (!prm.dbuf && next < prm.items) stage_item(next, 0);   // the strip buffer is free: refill it now
 
         quantize_item<P, GSR, SPLIT>(Zs, CBP, ntile, ng, gs, srow, tw0, c_base, g, tab, Xq, sX);
-        __syncthreads();   // Z and this strip buffer are free again
-    }
-}
-
-// ---- the fully quantized input transform (Eq. quant-B) ------------------------------------
-//   X~ = s_qB^2 s_qx  Q(S_B V_B / s_qB)  Q(x / s_qx)  Q(V_B^T S_B / s_qB)
-// with one s_qx per (tile, channel group) over the group's n x n patches; fp32(X~) is what the group
-// quantizer of the contraction's operand sees.  Work items, staging and quantization are those of
-// the kernel above; in between every (tile, channel) first contributes its patch to the abs-max of its
-// 32 channels (one warp reduction), then quantizes the patch (code_of_float) and forms the two
-// integer products.  32x32 C=640 F(4,3), two images: 15.5 us (latency of
-// the phases at 16 warps per SM, 45 % of the issue slots); with one CTA per (tile, group), each thread
-// reading its patch element by element from global memory (32 rows of memory per load instruction)
-// and all codes decided in fp64, 24.8 us.
-template <int M, typename Tin, int GSR, int SPLIT>
-__global__ void __launch_bounds__(K1_THREADS, 4)
-input_transform_int_kernel(const Tin *__restrict__ x, int8_t *__restrict__ Xq, float *__restrict__ sX, Geometry g,
-                           const __grid_constant__ FullQuantTables tab, K1Params prm)
-{
-    constexpr int NN = M + 2;
-    constexpr int P = NN * NN;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ float amax_s[(K1_WP - 3) / M][8];               // [tile][run of 32 channels]
-    ptx::grid_dependency_wait();
-    ptx::grid_launch_dependents();
-    float *Zs = reinterpret_cast<float *>(smem_raw + (1 + prm.dbuf) * prm.strip_bytes);   // [tile][position][CBP]
-    const int CBP = prm.CB + 4;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    constexpr int NWARP = K1_THREADS / 32;
-    const int cb32 = prm.CB >> 5;
-    const int gs = GSR > 0 ? GSR * SPLIT : g.gs;
-    const int ng = prm.CB / gs, gs32 = gs >> 5;
-
-    auto stage_item = [&](int item, int buf) {
-        const int cblk = item % prm.NCB, rest = item / prm.NCB;
-        const int srow = rest / prm.NCH, chunk = rest - srow * prm.NCH;
-        const int img = srow / g.TH, th = srow - img * g.TH;
-        const int first = chunk * prm.TB * M - 1;
-        const int w_base = prm.vec16 ? ((first + 8) & ~7) - 8 : first - 1;
-        stage_strip<Tin, NN>(reinterpret_cast<Tin *>(smem_raw + buf * prm.strip_bytes), x, g, prm, img,
-                             cblk * prm.CB, th * M - 1, w_base);
-        cp_async_commit();
-    };
-
-    int item = blockIdx.x;
-    if (prm.dbuf && item < prm.items) stage_item(item, 0);
-    for (int it = 0; item < prm.items; ++it, item += gridDim.x) {
-        const int buf = prm.dbuf ? (it & 1) : 0;
-        const int next = item + gridDim.x;
-        if (!prm.dbuf) {
-            if (it == 0) stage_item(item, 0);
-            cp_async_wait_group<0>();
-        } else if (next < prm.items) {
-            stage_item(next, buf ^ 1);
-            cp_async_wait_group<1>();
-        } else {
-            cp_async_wait_group<0>();
-        }
-        __syncthreads();
-
-        const Tin *strip = reinterpret_cast<const Tin *>(smem_raw + buf * prm.strip_bytes);
-        const int cblk = item % prm.NCB, rest = item / prm.NCB;
-        const int srow = rest / prm.NCH, chunk = rest - srow * prm.NCH;   // srow = img*TH + th
-        const int tw0 = chunk * prm.TB;
-        const int ntile = min(prm.TB, g.TW - tw0);
-        const int c_base = cblk * prm.CB;
-        const int voff = tw0 * M - 2 - (((tw0 * M - 1 + 8) & ~7) - 8);
-        auto patch = [&](int tl, int c, float (&d)[NN][NN]) {
-            if (sizeof(Tin) == 2 && prm.vec16) load_patch_vec<NN>(strip + c * prm.CS, tl * M + voff, d);
-            else load_patch<NN>(strip + c * prm.CS, tl * M, d);
-        };
-
-        for (int wt = warp; wt < ntile * cb32; wt += NWARP) {
-            const int tl = wt / cb32, c32 = wt - tl * cb32;
-            float d[NN][NN], m = 0.f;
-            patch(tl, c32 * 32 + lane, d);
-#pragma unroll
-            for (int a = 0; a < NN; ++a)
-#pragma unroll
-                for (int b = 0; b < NN; ++b) m = fmaxf(m, fabsf(d[a][b]));     // ignores NaN
-            const unsigned top = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
-            if (lane == 0) amax_s[tl][c32] = __uint_as_float(top);
-        }
-        __syncthreads();
-        for (int wt = warp; wt < ntile * cb32; wt += NWARP) {
-            const int tl = wt / cb32, c32 = wt - tl * cb32;
-            const int c = c32 * 32 + lane;
-            float amax = 0.f;                                    // of the group of these 32 channels
-            for (int k = c32 / gs32 * gs32, e = k + gs32; k < e; ++k) amax = fmaxf(amax, amax_s[tl][k]);
-            float d[NN][NN];
-            patch(tl, c, d);
-            const float rinv = __fdiv_rn(127.f, amax);
-            int q[NN][NN], tmp[NN][NN];
-#pragma unroll
-            for (int a = 0; a < NN; ++a)
-#pragma unroll
-                for (int b = 0; b < NN; ++b) q[a][b] = code_of_float(d[a][b], amax, rinv);
-#pragma unroll
-            for (int b = 0; b < NN; ++b)
-#pragma unroll
-                for (int i = 0; i < NN; ++i) {
-                    int s = 0;
-#pragma unroll
-                    for (int a = 0; a < NN; ++a) s += tab.BTq[i * NN + a] * q[a][b];
-                    tmp[i][b] = s;
-                }
-            const double scale = __dmul_rn(tab.sqB2, __ddiv_rn((double)amax, kIntQmax));
-            float *out = Zs + (size_t)tl * P * CBP + c;
-#pragma unroll
-            for (int i = 0; i < NN; ++i)
-#pragma unroll
-                for (int j = 0; j < NN; ++j) {
-                    int s = 0;
-#pragma unroll
-                    for (int b = 0; b < NN; ++b) s += tmp[i][b] * tab.BTq[j * NN + b];
-                    out[(i * NN + j) * CBP] = (float)__dmul_rn((double)s, scale);
-                }
-        }
-        __syncthreads();
-        if (!prm.dbuf && next < prm.items) stage_item(next, 0);   // the strip buffer is free: refill it now
-
-        quantize_item<P, GSR, SPLIT, false>(Zs, CBP, ntile, ng, gs, srow, tw0, c_base, g, ScaleTables{}, Xq, sX);
         __syncthreads();   // Z and this strip buffer are free again
     }
 }
@@ -827,41 +394,6 @@ cudaError_t launch_k1(const wfq_plan &plan, const void *x_dev, cudaStream_t stre
 }
 
 template <int M, typename Tin, int GSR, int SPLIT>
-int k1i_resident(size_t smem)
-{
-    return resident_ctas_per_sm(input_transform_int_kernel<M, Tin, GSR, SPLIT>, K1_THREADS, smem, 32);
-}
-
-template <int M, typename Tin, int GSR, int SPLIT>
-cudaError_t k1i_setup()
-{
-    auto kern = input_transform_int_kernel<M, Tin, GSR, SPLIT>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                (int)cudaSharedmemCarveoutMaxShared);
-}
-
-template <int M, typename Tin, int GSR, int SPLIT>
-cudaError_t launch_k1i(const wfq_plan &plan, const void *x_dev, cudaStream_t stream)
-{
-    const bool vec = plan.k1iv.vec16 && plan.k1_choice != 3 && (reinterpret_cast<uintptr_t>(x_dev) & 15u) == 0;
-    const K1Params &prm = vec ? plan.k1iv : plan.k1i;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)prm.grid);
-    cfg.blockDim = dim3(K1_THREADS);
-    cfg.dynamicSmemBytes = prm.smem;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, input_transform_int_kernel<M, Tin, GSR, SPLIT>, static_cast<const Tin *>(x_dev),
-                              plan.ws.Xq, plan.ws.sX, plan.geo, plan.fq, prm);
-}
-
-template <int M, typename Tin, int GSR, int SPLIT>
 int k1n_resident(size_t smem)
 {
     return resident_ctas_per_sm(input_transform_nhwc_kernel<M, Tin, GSR, SPLIT>, K1_THREADS, smem, 32);
@@ -896,7 +428,7 @@ cudaError_t launch_k1n(const wfq_plan &plan, cudaStream_t stream)
 }
 
 // What to do with the instantiation that serves (m, dtype, group size).
-enum K1Op { kK1Launch, kK1Resident, kK1Setup, kK1iLaunch, kK1iResident, kK1iSetup, kK1nLaunch, kK1nResident, kK1nSetup };
+enum K1Op { kK1Launch, kK1Resident, kK1Setup, kK1nLaunch, kK1nResident, kK1nSetup };
 
 template <int M, typename Tin>
 long long k1_by_gs(K1Op op, int gs, const wfq_plan *plan, const void *x, cudaStream_t s, size_t smem)
@@ -906,9 +438,6 @@ long long k1_by_gs(K1Op op, int gs, const wfq_plan *plan, const void *x, cudaStr
         case kK1Launch: return (long long)launch_k1<M, Tin, GSR, SPLIT>(*plan, x, s);  \
         case kK1Resident: return k1_resident<M, Tin, GSR, SPLIT>(smem);                \
         case kK1Setup: return (long long)k1_setup<M, Tin, GSR, SPLIT>();               \
-        case kK1iLaunch: return (long long)launch_k1i<M, Tin, GSR, SPLIT>(*plan, x, s); \
-        case kK1iResident: return k1i_resident<M, Tin, GSR, SPLIT>(smem);              \
-        case kK1iSetup: return (long long)k1i_setup<M, Tin, GSR, SPLIT>();             \
         case kK1nLaunch: return (long long)launch_k1n<M, Tin, GSR, SPLIT>(*plan, s);   \
         case kK1nResident: return k1n_resident<M, Tin, GSR, SPLIT>(smem);              \
         default: return (long long)k1n_setup<M, Tin, GSR, SPLIT>();                    \
@@ -933,9 +462,7 @@ long long k1_op(K1Op op, int m, bool f16, int gs, const wfq_plan *plan, const vo
 
 }  // namespace
 
-namespace {
-
-void plan_k1(wfq_plan &plan, K1Params &prm, bool vec16, K1Op resident_op)
+void plan_k1(wfq_plan &plan, K1Params &prm, bool vec16, ResidentFn resident_of)
 {
     const Geometry &g = plan.geo;
     const bool f16 = plan.in_dtype == WFQ_F16;
@@ -974,12 +501,10 @@ void plan_k1(wfq_plan &plan, K1Params &prm, bool vec16, K1Op resident_op)
     prm.NCB = g.C / prm.CB;
     prm.items = g.N * g.TH * prm.NCH * prm.NCB;
     // persistent CTAs: as many as fit on the device at once
-    const int per_sm = (int)k1_op(resident_op, M, f16, g.gs, nullptr, nullptr, nullptr, (size_t)prm.smem);
+    const int per_sm = resident_of(plan, (size_t)prm.smem);
     const int resident = per_sm * (plan.sm_count > 0 ? plan.sm_count : 1);
     prm.grid = prm.items < resident ? prm.items : resident;
 }
-
-}  // namespace
 
 // The same for the NHWC kernel: the strip is the dense TMA box [n][TB * m + 2][CB].
 static void plan_k1_nhwc(wfq_plan &plan)
@@ -1024,12 +549,12 @@ static void plan_k1_nhwc(wfq_plan &plan)
 void plan_input_transform(wfq_plan &plan)
 {
     const bool vec16 = plan.in_dtype == WFQ_F16 && plan.geo.W % 8 == 0;
-    plan_k1(plan, plan.k1, false, kK1Resident);
+    auto resident_of = [](const wfq_plan &p, size_t smem) {
+        return (int)k1_op(kK1Resident, p.geo.m, p.in_dtype == WFQ_F16, p.geo.gs, nullptr, nullptr, nullptr, smem);
+    };
+    plan_k1(plan, plan.k1, false, resident_of);
     plan.k1v = plan.k1;
-    if (vec16) plan_k1(plan, plan.k1v, true, kK1Resident);
-    plan_k1(plan, plan.k1i, false, kK1iResident);
-    plan.k1iv = plan.k1i;
-    if (vec16) plan_k1(plan, plan.k1iv, true, kK1iResident);
+    if (vec16) plan_k1(plan, plan.k1v, true, resident_of);
     plan_k1_nhwc(plan);
     plan.tmap_xn_base = nullptr;
     plan.tmap_xn_tc_base = nullptr;
@@ -1043,18 +568,10 @@ cudaError_t setup_input_transform()
             for (int gs : sizes) {
                 cudaError_t e = (cudaError_t)k1_op(kK1Setup, m, f16 != 0, gs, nullptr, nullptr, nullptr, 0);
                 if (e != cudaSuccess) return e;
-                e = (cudaError_t)k1_op(kK1iSetup, m, f16 != 0, gs, nullptr, nullptr, nullptr, 0);
-                if (e != cudaSuccess) return e;
                 e = (cudaError_t)k1_op(kK1nSetup, m, f16 != 0, gs, nullptr, nullptr, nullptr, 0);
                 if (e != cudaSuccess) return e;
             }
     return cudaSuccess;
-}
-
-// The fully quantized input transform (NCHW input, any group size of the plan).
-cudaError_t launch_input_transform_int(const wfq_plan &plan, const void *x_dev, cudaStream_t stream)
-{
-    return (cudaError_t)k1_op(kK1iLaunch, plan.geo.m, plan.in_dtype == WFQ_F16, plan.geo.gs, &plan, x_dev, stream, 0);
 }
 
 cudaError_t launch_input_transform(wfq_plan &plan, const void *x_dev, cudaStream_t stream)

@@ -123,7 +123,7 @@ struct wfq_plan {
     // launch parameters derived from the geometry, the dtype and the device (plan_launches)
     wfq::K1Params k1;          // 4-byte (or 2-byte) copies: any x
     wfq::K1Params k1v;         // 16-byte copies where the layer allows them (vec16 set), else a copy of k1
-    wfq::K1Params k1i, k1iv;   // the same two for the fully quantized input transform
+    wfq::K1Params k1i, k1iv;   // the same two for the fully quantized input transform (set while fq_input is)
     wfq::K1Params k1n;         // NHWC input: one TMA box per work item
     bool in_nhwc = false;      // x is [N][H][W][C] instead of [N][C][H][W]
     CUtensorMap tmap_xn;       // the NHWC input as (C, W, H, N)
@@ -192,6 +192,9 @@ bool encode_tmap(CUtensorMap *map, CUtensorMapDataType dtype, int rank, const vo
 cudaError_t launch_gemm(const wfq_plan &plan, int32_t *acc_dump, cudaStream_t stream, bool pdl);
 cudaError_t launch_output_transform(const wfq_plan &plan, float *y_dev, cudaStream_t stream, bool pdl);
 void build_full_quant_tables(wfq_plan &plan);
+cudaError_t plan_input_transform_int(wfq_plan &plan);
+using ResidentFn = int (*)(const wfq_plan &plan, size_t smem);   // CTAs per SM of the plan's kernel
+void plan_k1(wfq_plan &plan, K1Params &prm, bool vec16, ResidentFn resident_of);
 cudaError_t launch_input_transform_int(const wfq_plan &plan, const void *x_dev, cudaStream_t stream);
 cudaError_t launch_output_transform_int(const wfq_plan &plan, float *y_dev, cudaStream_t stream, bool pdl);
 cudaError_t launch_mma_peak(const wfq_plan &plan, int n_cols, int mmas, cudaStream_t stream);
