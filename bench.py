@@ -10,7 +10,9 @@ direct-convolution-equivalent throughput, 2*N*K*C*H*W*9 operations per layer div
 by the time of the forward call (filter preparation is offline and not timed).  The
 headline workload is configuration 5, the largest one (the full UNet conv-layer set).
 
-One JSON line is printed by rank 0.  Besides the throughput it carries
+One JSON line is printed by rank 0 on stdout, short enough to survive where only the end of a program's output is
+kept: the throughput and, of the blocks below, the figures themselves.  The whole record goes to stderr as
+one JSON line before it (`details`); it carries
   roofline      achieved HBM GB/s of the kernel that takes the most time in a step,
                 from CUDA events around the chain prefixes K1, K1+K2, K1+K2+K3
   per_config    the same figures for each of the five configurations (fewer steps)
@@ -251,6 +253,44 @@ def run_reference(args):
             "e2e": {"value": value, "unit": UNIT, "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0},
             "gpu_launches": 0}
     print(json.dumps(line), flush=True)
+
+
+# ---- the printed line ------------------------------------------------------------------
+LINE_LIMIT = 2500          # characters
+
+
+def _part(block, keys):
+    return None if block is None else {k: block[k] for k in keys if k in block}
+
+
+def _values(blocks):
+    return {name: b_["error"] if "error" in b_ else b_["value"] for name, b_ in (blocks or {}).items() if b_ is not None}
+
+
+def printed_line(record):
+    """The stdout line of a record: every scalar and `config` whole, of the other blocks the figures themselves."""
+    line = {k: v for k, v in record.items() if not isinstance(v, (dict, list))}
+    line["config"] = record["config"]
+    line["clocks"] = record.get("clocks")
+    line["e2e"] = _part(record.get("e2e"), ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "steps",
+                                            "matches_synchronous_result"))
+    line["roofline"] = _part(record.get("roofline"), ("bound", "kernel", "achieved", "peak", "unit", "frac", "traffic",
+                                                      "launches_per_step", "algorithmic_bytes_per_launch", "us_per_launch"))
+    line["parity"] = _part(record.get("parity"), ("ok", "worst_rel_err", "tolerance", "int8_code_mismatch_rate"))
+    line["cpu_baseline"] = _part(record.get("cpu_baseline"), ("value", "unit", "cores", "kind"))
+    line["us_per_step"] = {name: _part(record.get(name), ("us_per_step",)).get("us_per_step")
+                           for name in ("nhwc_input", "layers_on_three_streams", "w4_weights") if record.get(name)}
+    line["values"] = dict(_values(record.get("per_config")), **_values(record.get("full_quant")))
+    for k in ("us_per_step", "values"):
+        if not line[k]:
+            del line[k]
+    text = json.dumps(line)
+    for k in ("values", "us_per_step", "cpu_baseline", "parity", "roofline"):     # least needed first
+        if len(text) <= LINE_LIMIT:
+            break
+        line.pop(k, None)
+        text = json.dumps(line)
+    return text
 
 
 # ---- aggregation over replicas ---------------------------------------------------------
@@ -821,8 +861,8 @@ def run_wfq(args):
                 full_quant[label] = {"workload": s3["workload"], "value": s3["value"], "unit": UNIT,
                                      "us_per_step": s3["us_per_step"], "kernels": s3["kernels"],
                                      "us_per_layer": s3["us_per_layer"], "parity": w3.parity_full_quant(y_scale),
-                                     "note": "integer input and output transforms (Eqs. quant-B, quant-y), "
-                                             "reference-speed kernels; same contraction kernel"}
+                                     "note": "integer input and output transforms (Eqs. quant-B, quant-y); "
+                                             "same contraction kernel"}
                 w3.close()
                 del w3
                 torch.cuda.empty_cache()
@@ -925,7 +965,8 @@ def run_wfq(args):
                 "warm": warm, "sustained": sustained, "roofline": roofline, "contraction": contraction,
                 "parity": parity, "per_config": per_config, "full_quant": full_quant, "nhwc_input": nhwc, "layers_on_three_streams": concurrent, "w4_weights": w4, "cpu_baseline": cpu, "e2e": e2e,
                 "gpu_launches": 3 * len(layers) * args.steps * reps, "clocks": clocks}
-        print(json.dumps(line), flush=True)
+        print("details " + json.dumps(line), file=sys.stderr, flush=True)
+        print(printed_line(line), flush=True)
     if world > 1:
         dist.barrier()
         dist.destroy_process_group()
