@@ -58,7 +58,7 @@ typedef enum {
     WFQ_ERR_NOT_PREPARED = 4, /* workspace or filters missing */
     WFQ_ERR_CUDA = 5,         /* a CUDA runtime/driver call failed */
     WFQ_ERR_TIMEOUT = 6,      /* a bounded device-side wait expired (status word) */
-    WFQ_ERR_SCRATCH_TOO_SMALL = 7 /* problem larger than the library's built-in scratch */
+    WFQ_ERR_SCRATCH_TOO_SMALL = 7 /* beyond the size limit of wfq_quantize_filters_static */
 } wfq_status_t;
 
 typedef enum { WFQ_F32 = 0, WFQ_F16 = 1, WFQ_BF16 = 2 /* output only */ } wfq_dtype_t;
@@ -177,7 +177,9 @@ wfq_status_t wfq_plan_set_weight_bits(wfq_plan_t *plan, int bits);
  * With an integer output transform the scale vectors given to wfq_prepare_filters change the
  * result (this is where the paper's learned scales act); with the floating-point transforms they
  * are numerically neutral.  Group sizes: multiples of 32 up to 256.  Host only; takes effect from
- * the next forward call.
+ * the next forward call.  Where the plan has its workspace, the call that switches quant_input on
+ * sets the attributes of its kernel (the first one in a process also loads it); otherwise
+ * wfq_plan_set_workspace does.
  */
 typedef enum { WFQ_Y_FP32 = 0, WFQ_Y_TILE = 1, WFQ_Y_ROW = 2 } wfq_y_quant_t;
 wfq_status_t wfq_plan_set_full_quant(wfq_plan_t *plan, int quant_input, wfq_y_quant_t y_mode);
@@ -209,10 +211,10 @@ wfq_status_t wfq_plan_set_workspace(wfq_plan_t *plan, void *dev_ptr, size_t byte
  *            evaluated in fp64 and rounded to fp32)
  * All scales must be finite and nonzero (signs are allowed).  The first call on a plan
  * allocates the plan-owned Wq/sW buffers and the status word with cudaMalloc (which may
- * synchronise the device); every call takes the fp32 temporary between its two kernels
- * from the stream-ordered allocator (cudaMallocAsync / cudaFreeAsync on `stream`), so
- * later calls neither block nor synchronise.  Asynchronous on `stream`; may be called
- * again to replace the filters.  The first library call that meets a device (this one or
+ * synchronise the device); otherwise a call is one kernel without temporaries, so later
+ * calls neither block nor synchronise.  Asynchronous on `stream`; may be called
+ * again to replace the filters, and a forward call may follow on the same stream with
+ * nothing in between.  The first library call that meets a device (this one or
  * wfq_plan_set_workspace) also sets that device's kernel attributes; make it outside any
  * stream capture.
  */
@@ -239,7 +241,8 @@ wfq_status_t wfq_prepare_filters(wfq_plan_t *plan, const float *w_dev, const flo
  *   m in {2,4,6}; group_size a multiple of 32, at most 256, dividing C.
  *
  * Limit: (m+2)^2 * K * C <= WFQ_STATIC_SCRATCH_FLOATS, otherwise
- * WFQ_ERR_SCRATCH_TOO_SMALL is returned and nothing is launched.  Other argument errors
+ * WFQ_ERR_SCRATCH_TOO_SMALL is returned and nothing is launched (the names are older than
+ * the kernel, which needs no scratch: the limit is kept for callers that rely on it).  Other argument errors
  * are reported as in wfq_prepare_filters.  Asynchronous on `stream`.
  *
  * Calls share nothing: they may overlap on different streams and from different threads.

@@ -149,7 +149,7 @@ const char *wfq_status_string(wfq_status_t s)
         case WFQ_ERR_CUDA: return "CUDA call failed";
         case WFQ_ERR_TIMEOUT: return "device-side wait timed out";
         case WFQ_ERR_SCRATCH_TOO_SMALL:
-            return "problem exceeds the library's built-in scratch array";
+            return "problem exceeds the size limit of the allocation-free filter quantization";
     }
     return "unknown status";
 }

@@ -157,7 +157,9 @@ __device__ __forceinline__ void store_tiles(const RowOf &row_of, StoreShared<M, 
 // tiles of 128 channels with an epilogue (36.4 -> 33.7 us), 162 of 256 (26.6 -> 25.9 us).  With about
 // the same number of threads they are no better (121 tiles of 640 channels 41.2 -> 41.8 us, 3200 and 1600
 // tiles within 0.3 us), and F(4,3) and F(2,3) gain nothing from them (32 tiles of 1280 channels 26.5 ->
-// 26.8 us, 3136 tiles of 128 channels 23.9 -> 24.4 us).
+// 26.8 us, 3136 tiles of 128 channels 23.9 -> 24.4 us).  The integer kernels gain more: forward with one scale
+// per tile, 36 tiles of 640 channels 28.6 -> 26.3 us, with one per row 48.5 -> 34.1 us; 800 tiles of 64
+// channels 30.9 -> 29.9 and 50.1 -> 37.3 us.
 bool half_ctas(const Geometry &g)
 {
     const long long by64 = ((long long)g.T + 63) / 64 * 64, by128 = ((long long)g.T + 127) / 128 * 128;

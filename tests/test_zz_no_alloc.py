@@ -2,10 +2,9 @@
 
 Hosts that cannot call cudaMalloc when filters arrive (a framework whose pool owns the
 device, a latency-critical loop, a fixed memory budget) use
-wfq_quantize_filters_static, which keeps its intermediate in an array built into the
-library.  Both entry points must give the same codes and scales; the built-in array is
-shared by all calls, so two calls in a row (the second on a smaller layer, which leaves
-the first call's values behind in the array) are both checked.  This file is collected
+wfq_quantize_filters_static, which writes into the caller's buffers and keeps nothing.
+Both entry points must give the same codes and scales, also for two layers one after the
+other, and requests above the size limit are refused.  This file is collected
 last on purpose: a failure here must not hide the results of the other tests.
 """
 import numpy as np
