@@ -27,7 +27,9 @@ struct FilterTables {
 // Bound: latency of about ten dependent instructions per transformed value (3-4 of them fp64) at the 12 warps
 // per SM that the filters of four channels in fp64 leave room for: 2.2 of 4 issue slots per cycle and SM are
 // used.  Nothing but w, Wq and sW touches memory.  640 -> 1280 channels, F(6,3), groups of 64 (82 MB in and
-// out, 13 us at 6.55 TB/s): 45 us alone, 47 us back to back.  The former pair of kernels (one thread per filter, then one thread per group
+// out, 13 us at 6.55 TB/s): 45 us alone, 47 us back to back.  Groups above 128 hold twice the filters per lane (two
+// CTAs per SM, 28 bytes spilled): 1280 -> 640 channels, groups of 256, 64 us; groups of 160, whose second run of lanes
+// is three quarters empty, 640 -> 1280 channels 92 us.  The former pair of kernels (one thread per filter, then one thread per group
 // reading serially, through an fp32 array four times the size of Wq taken from the stream-ordered
 // allocator) took 690 us, and 20 ms when the device was idle in between and the pool had been given back.
 constexpr int FP_WARPS = 4;       // warps per CTA
