@@ -163,8 +163,7 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     constexpr int CW = C::CW;
     extern __shared__ unsigned char smem_raw[];
     // 1024-byte alignment: the 128-byte swizzle atoms repeat every 1024 bytes
-    unsigned char *tiles = reinterpret_cast<unsigned char *>(
-        (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    unsigned char *tiles = ptx::align_smem<1024>(smem_raw);
     float *scales = reinterpret_cast<float *>(tiles + (size_t)NSTAGES * C::STAGE_BYTES);
     Shared *sh = reinterpret_cast<Shared *>(scales + (size_t)NSLOT * C::SLOT_SCALE_FLOATS);
 
@@ -572,8 +571,7 @@ template <int BN>
 __global__ void __launch_bounds__(128, 1) mma_peak_kernel(int mmas, int *status, long long wait_cycles)
 {
     extern __shared__ unsigned char smem_raw[];
-    unsigned char *tiles = reinterpret_cast<unsigned char *>(
-        (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    unsigned char *tiles = ptx::align_smem<1024>(smem_raw);
     constexpr int BYTES = (BM + BN) * BK;
     PeakShared *sh = reinterpret_cast<PeakShared *>(tiles + BYTES);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;

@@ -268,8 +268,7 @@ input_transform_nhwc_kernel(const __grid_constant__ CUtensorMap tmx, int8_t *__r
     __shared__ K1NhwcShared sh;
     // a TMA destination must be 128-byte aligned; the dynamic part starts wherever the static part
     // ends, so the strips start at the next multiple of 128 (the launch adds 128 bytes for this)
-    unsigned char *smem_raw = reinterpret_cast<unsigned char *>(
-        (reinterpret_cast<uintptr_t>(smem_dyn) + 127) & ~(uintptr_t)127);
+    unsigned char *smem_raw = ptx::align_smem<128>(smem_dyn);
     ptx::grid_dependency_wait();
     ptx::grid_launch_dependents();
     float *Zs = reinterpret_cast<float *>(smem_raw + (1 + prm.dbuf) * prm.strip_bytes);   // [tile][position][CBP]

@@ -189,8 +189,7 @@ input_transform_tc_kernel(const __grid_constant__ CUtensorMap tmx, TcArgs a, Geo
     using C = TcCfg<M>;
     constexpr int NN = C::NN, P = C::P, S = C::S, PL = C::PL, KSTEPS = C::KSTEPS;
     extern __shared__ unsigned char smem_raw[];
-    unsigned char *base = reinterpret_cast<unsigned char *>(
-        (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    unsigned char *base = ptx::align_smem<1024>(smem_raw);
     unsigned char *Bring = base;                                 // [2 * nbp][64 rows][128 B]
     unsigned char *strips = Bring + (size_t)2 * a.nbp * TC_TILE_BYTES;
     TcShared *sh = reinterpret_cast<TcShared *>(strips + (size_t)a.nstrip * a.strip_bytes);

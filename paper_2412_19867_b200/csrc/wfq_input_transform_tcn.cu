@@ -112,8 +112,7 @@ input_transform_tcn_kernel(const __grid_constant__ CUtensorMap tmx, TnArgs a, Ge
     constexpr int TN_NSTRIP = C::NSTRIP, TN_NACC = C::NACC, TN_TEAMS = C::TEAMS, TN_THREADS = C::THREADS;
     extern __shared__ unsigned char smem_dyn[];
     __shared__ TnShared sh;
-    unsigned char *base = reinterpret_cast<unsigned char *>(
-        (reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~(uintptr_t)1023);     // swizzle atoms repeat every 1024 B
+    unsigned char *base = ptx::align_smem<1024>(smem_dyn);     // swizzle atoms repeat every 1024 B
     unsigned char *amat_s = base;
     unsigned char *strips = base + C::A_BYTES;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;

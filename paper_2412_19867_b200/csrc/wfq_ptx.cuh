@@ -14,6 +14,15 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p)
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// The next multiple of A at or behind p, as an offset from p: rounded as an integer the pointer would lose its address
+// space, and every access through it would be a generic one (the contraction's scale loads: 14x14 with groups of 32,
+// 64 images, 44.7 -> 43.6 us forward, 1280 channels 32x32 45.7 -> 44.4 us, ten layers 1.7 % less time).
+template <uint32_t A>
+__device__ __forceinline__ unsigned char *align_smem(unsigned char *p)
+{
+    return p + (-smem_u32(p) & (A - 1u));
+}
+
 // ---- mbarrier -----------------------------------------------------------------------
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count)
 {
