@@ -18,7 +18,7 @@
 //            instruction): waits for a stage and, at the start of a chunk, for its TMEM
 //            slot; commits the stage back to the producer and the chunk to the epilogue
 //   warp 2   scale loader: per chunk, 128 row scales and BN column scales per group into
-//            the chunk's scale slot (bulk copies)
+//            the chunk's scale slot (bulk copies); their arrival counts on the same barrier as the MMAs'
 //   warps 4-7   epilogue: warp % 4 selects the 32 TMEM lanes the warp may read; each warp
 //            handles all BN columns of its lanes.  Per chunk: wait for accumulators and
 //            scales, then per group tcgen05.ld the int32 sums, convert and scale into fp32
@@ -41,34 +41,36 @@ namespace {
 constexpr int BM = 128;        // rows per unit (MMA M, TMEM lanes)
 constexpr int BK = 128;        // bytes (= int8 channels) per pipeline stage
 constexpr int UK = 32;         // channels per MMA instruction
-constexpr int NSTAGES = 4;     // shared-memory operand stages
+constexpr int NSTAGES = 3;     // shared-memory operand stages
 constexpr int NSLOT = 2;       // TMEM / scale slots (chunks in flight)
 constexpr int SLOT_COLS = 128; // TMEM columns per slot
 constexpr int TMEM_COLS = NSLOT * SLOT_COLS;
 constexpr int A_BYTES = BM * BK;
-constexpr int NUM_EPI_WARPS = 4;
+constexpr int NUM_EPI_WARPS = 4;   // one per 32 TMEM lanes
 constexpr int FIRST_EPI_WARP = 4;
 constexpr int NUM_THREADS = 32 * (FIRST_EPI_WARP + NUM_EPI_WARPS);
 
 struct Shared {
-    uint64_t full[NSTAGES];        // operands of a stage have landed
-    uint64_t empty[NSTAGES];       // the MMAs reading a stage have completed
-    uint64_t acc_full[NSLOT];      // the MMAs of a chunk have completed
+    uint64_t full[NSTAGES];     // operands of a stage have landed
+    uint64_t empty[NSTAGES];    // the MMAs reading a stage have completed
+    uint64_t acc_full[NSLOT];      // the MMAs of a chunk have completed and its scales have landed
     uint64_t slot_free[NSLOT];     // all epilogue warps are done with a chunk
-    uint64_t scale_full[NSLOT];    // the scales of a chunk have landed
     uint32_t tmem_base;
     volatile int abort;
 };
 
-template <int BN>
+// Normal orientation: the epilogue hands Y to the TMA unit through shared memory.  Three stages leave the room for it and
+// are no slower than four (forward, ten layers within 0.2 %; swapped, 36 tiles x 1280 channels F(6,3) 44.0 -> 43.6 us).
+template <int BN, bool SWAP>
 struct Cfg {
+    static constexpr int STORE_BYTES = SWAP ? 0 : BM * BN * 4;
     static constexpr int B_BYTES = BN * BK;
     static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
     static constexpr int CG_MAX = SLOT_COLS / BN;             // groups per chunk at most
     static constexpr int GROUP_SCALE_FLOATS = BM + BN;        // row scales, then column scales
     static constexpr int SLOT_SCALE_FLOATS = CG_MAX * GROUP_SCALE_FLOATS;
-    static constexpr int CW = BN / (NUM_EPI_WARPS / 4);       // columns per epilogue warp
-    static constexpr size_t SMEM_BYTES = 1024 /*alignment slack*/ + (size_t)NSTAGES * STAGE_BYTES +
+    static constexpr int CW = BN;                             // columns per epilogue warp
+    static constexpr size_t SMEM_BYTES = 1024 /*alignment slack*/ + (size_t)NSTAGES * STAGE_BYTES + STORE_BYTES +
                                          (size_t)NSLOT * SLOT_SCALE_FLOATS * sizeof(float) + sizeof(Shared);
 };
 
@@ -92,12 +94,12 @@ struct GemmArgs {
 // descriptor offsets and accumulate flags, one commit.  The generic loop in the kernel
 // spends several hundred cycles per MMA on its bookkeeping, which made the issuing
 // warp the bottleneck of every layer with more than one chunk per unit.
-template <int BN, int GSTEPS, int CGT>
+template <int BN, bool SWAP, int GSTEPS, int CGT>
 __device__ __forceinline__ void mma_issue_aligned(Shared *sh, uint32_t tiles_lo, uint32_t tmem_base,
                                                   int units, int KB, int last_slices, int lane,
                                                   const WaitCtx &ctx)
 {
-    using C = Cfg<BN>;
+    using C = Cfg<BN, SWAP>;
     constexpr int CHUNK_STEPS = GSTEPS * CGT;            // MMAs per chunk
     constexpr int NCH = (BK / UK) / CHUNK_STEPS;         // chunks per stage
     static_assert(NCH >= 1 && NCH * CHUNK_STEPS == BK / UK, "chunks must tile a stage");
@@ -121,7 +123,7 @@ __device__ __forceinline__ void mma_issue_aligned(Shared *sh, uint32_t tiles_lo,
                                                               kWaitTmemEmpty)))
                         return;
                     ptx::tc_fence_after();
-                    if (lane == 0) {
+                    if (ptx::elect_one()) {
                         const uint32_t d = tmem_base + (uint32_t)(slot * SLOT_COLS);
                         if ((c + 1) * CHUNK_STEPS <= nslice) {
 #pragma unroll
@@ -147,7 +149,7 @@ __device__ __forceinline__ void mma_issue_aligned(Shared *sh, uint32_t tiles_lo,
                     if (++slot == NSLOT) { slot = 0; sphase ^= 1u; }
                 }
             }
-            if (lane == 0) ptx::umma_commit(empty0 + 8u * stage);
+            if (ptx::elect_one()) ptx::umma_commit(empty0 + 8u * stage);
             __syncwarp();
             if (++stage == NSTAGES) { stage = 0; phase ^= 1u; }
         }
@@ -157,14 +159,15 @@ __device__ __forceinline__ void mma_issue_aligned(Shared *sh, uint32_t tiles_lo,
 template <int BN, bool SWAP, bool DUMP>
 __global__ void __launch_bounds__(NUM_THREADS, 2)
 gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                    GemmArgs a, Geometry g)
+                    const __grid_constant__ CUtensorMap tmY, GemmArgs a, Geometry g)
 {
-    using C = Cfg<BN>;
+    using C = Cfg<BN, SWAP>;
     constexpr int CW = C::CW;
     extern __shared__ unsigned char smem_raw[];
     // 1024-byte alignment: the 128-byte swizzle atoms repeat every 1024 bytes
     unsigned char *tiles = ptx::align_smem<1024>(smem_raw);
-    float *scales = reinterpret_cast<float *>(tiles + (size_t)NSTAGES * C::STAGE_BYTES);
+    unsigned char *store = tiles + (size_t)NSTAGES * C::STAGE_BYTES;
+    float *scales = reinterpret_cast<float *>(store + C::STORE_BYTES);
     Shared *sh = reinterpret_cast<Shared *>(scales + (size_t)NSLOT * C::SLOT_SCALE_FLOATS);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -182,9 +185,8 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             ptx::mbar_init(ptx::smem_u32(&sh->empty[s]), 1);
         }
         for (int b = 0; b < NSLOT; ++b) {
-            ptx::mbar_init(ptx::smem_u32(&sh->acc_full[b]), 1);
+            ptx::mbar_init(ptx::smem_u32(&sh->acc_full[b]), DUMP ? 1 : 2);   // MMAs, scales
             ptx::mbar_init(ptx::smem_u32(&sh->slot_free[b]), NUM_EPI_WARPS);
-            ptx::mbar_init(ptx::smem_u32(&sh->scale_full[b]), 1);
         }
         sh->abort = 0;
         ptx::fence_mbar_init();
@@ -207,9 +209,10 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     constexpr int W_ROWS = SWAP ? BM : BN;                 // filter rows of a stage
     // stages of the first unit whose filter half is loaded early
     const int pre = (a.l2_prefetch_bytes > 0 && (int)blockIdx.x < units) ? (KB < NSTAGES ? KB : NSTAGES) : 0;
-    if (warp == 0 && lane == 0) {
+    if (warp == 0 && ptx::elect_one()) {
         ptx::prefetch_tmap(&tmA);
         ptx::prefetch_tmap(&tmB);
+        if (!SWAP) ptx::prefetch_tmap(&tmY);
         const CUtensorMap *tmW = SWAP ? &tmA : &tmB;
         long long budget = a.l2_prefetch_bytes;
         for (int u = blockIdx.x, first = 1; u < units && budget > 0; u += gridDim.x, first = 0) {
@@ -248,7 +251,7 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 ok = __all_sync(0xffffffffu, wait_bounded(ptx::smem_u32(&sh->empty[stage]), phase ^ 1u, ctx,
                                                           kWaitSmemEmpty));
                 if (!ok) break;
-                if (lane == 0 && !(blockIdx.x == 0 && issued == a.debug_skip_stage)) {
+                if (ptx::elect_one() && !(blockIdx.x == 0 && issued == a.debug_skip_stage)) {
                     const uint32_t bar = ptx::smem_u32(&sh->full[stage]);
                     const uint32_t a_dst = ptx::smem_u32(tiles + (size_t)stage * C::STAGE_BYTES);
                     if (issued >= pre) {
@@ -291,13 +294,13 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         bool ok = true;
         // shapes whose chunks tile a stage exactly take the straight-line issue loop
         if (gs_steps == 2 && cg == 2) {
-            mma_issue_aligned<BN, 2, 2>(sh, tiles_lo, tmem_base, units, KB, last_slices, lane, ctx);
+            mma_issue_aligned<BN, SWAP, 2, 2>(sh, tiles_lo, tmem_base, units, KB, last_slices, lane, ctx);
             ok = false;
         } else if (gs_steps == 4 && cg == 1) {
-            mma_issue_aligned<BN, 4, 1>(sh, tiles_lo, tmem_base, units, KB, last_slices, lane, ctx);
+            mma_issue_aligned<BN, SWAP, 4, 1>(sh, tiles_lo, tmem_base, units, KB, last_slices, lane, ctx);
             ok = false;
         } else if (gs_steps == 1 && cg == C::CG_MAX && C::CG_MAX <= 4) {
-            mma_issue_aligned<BN, 1, (C::CG_MAX <= 4 ? C::CG_MAX : 4)>(sh, tiles_lo, tmem_base, units, KB,
+            mma_issue_aligned<BN, SWAP, 1, (C::CG_MAX <= 4 ? C::CG_MAX : 4)>(sh, tiles_lo, tmem_base, units, KB,
                                                                     last_slices, lane, ctx);
             ok = false;
         }
@@ -323,26 +326,26 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                         ptx::tc_fence_after();
                         dcol = tmem_base + (uint32_t)(slot * SLOT_COLS);
                     }
-                    if (lane == 0) {
+                    if (ptx::elect_one()) {
                         if (in_group) ptx::umma_i8_lo<true>(dcol, a_lo + 2 * s, b_lo + 2 * s, dhi, idesc);
                         else ptx::umma_i8_lo<false>(dcol, a_lo + 2 * s, b_lo + 2 * s, dhi, idesc);
                     }
                     ++step;
                     if (++in_group == gs_steps) { in_group = 0; dcol += BN; }
                     if (step == chunk_steps) {
-                        if (lane == 0) ptx::umma_commit(ptx::smem_u32(&sh->acc_full[slot]));
+                        if (ptx::elect_one()) ptx::umma_commit(ptx::smem_u32(&sh->acc_full[slot]));
                         step = 0;
                         if (++slot == NSLOT) { slot = 0; sphase ^= 1u; }
                     }
                 }
                 if (!ok) break;
-                if (lane == 0) ptx::umma_commit(ptx::smem_u32(&sh->empty[stage]));
+                if (ptx::elect_one()) ptx::umma_commit(ptx::smem_u32(&sh->empty[stage]));
                 __syncwarp();
                 if (++stage == NSTAGES) { stage = 0; phase ^= 1u; }
             }
             if (ok && step != 0) {
                 // the last chunk of the unit has fewer groups than a full one
-                if (lane == 0) ptx::umma_commit(ptx::smem_u32(&sh->acc_full[slot]));
+                if (ptx::elect_one()) ptx::umma_commit(ptx::smem_u32(&sh->acc_full[slot]));
                 __syncwarp();
                 if (++slot == NSLOT) { slot = 0; sphase ^= 1u; }
             }
@@ -361,9 +364,9 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                     ok = __all_sync(0xffffffffu, wait_bounded(ptx::smem_u32(&sh->slot_free[slot]), sphase ^ 1u,
                                                               ctx, kWaitScaleEmpty));
                     if (!ok) break;
-                    const uint32_t bar = ptx::smem_u32(&sh->scale_full[slot]);
+                    const uint32_t bar = ptx::smem_u32(&sh->acc_full[slot]);
                     const uint32_t dst = ptx::smem_u32(scales + (size_t)slot * C::SLOT_SCALE_FLOATS);
-                    if (lane == 0) ptx::mbar_arrive_expect_tx(bar, (uint32_t)(ng * C::GROUP_SCALE_FLOATS * 4));
+                    if (ptx::elect_one()) ptx::mbar_arrive_expect_tx(bar, (uint32_t)(ng * C::GROUP_SCALE_FLOATS * 4));
                     __syncwarp();
                     // lane j copies the row scales of group j, lane 4 + j its column scales
                     if (lane < 8 && (lane & 3) < ng) {
@@ -386,7 +389,7 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 const long long n = issued < NSLOT ? issued : NSLOT;
                 for (long long i = 0; i < n; ++i) {
                     if (--s < 0) { s = NSLOT - 1; ph ^= 1u; }
-                    drain(ptx::smem_u32(&sh->scale_full[s]), ph, a.wait_cycles / 16);
+                    drain(ptx::smem_u32(&sh->acc_full[s]), ph, a.wait_cycles / 16);
                 }
             }
         }
@@ -414,10 +417,6 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 if (!wait_bounded(ptx::smem_u32(&sh->acc_full[slot]), sphase, ctx, kWaitTmemFull)) {
                     ok = false; break;
                 }
-                if constexpr (!DUMP) {
-                    if (!wait_bounded(ptx::smem_u32(&sh->scale_full[slot]), sphase, ctx,
-                                      kWaitScaleFull)) { ok = false; break; }
-                }
                 if (active) {
                     ptx::tc_fence_after();
                     const float *sc = scales + (size_t)slot * C::SLOT_SCALE_FLOATS;
@@ -427,11 +426,13 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                         const float2 rs2 = make_float2(rs, rs);
                         const float4 *cs4 = reinterpret_cast<const float4 *>(
                             sc + j * C::GROUP_SCALE_FLOATS + BM + c0);
+                        uint32_t rr[2][16];
+                        ptx::tmem_ld_x16(taddr, rr[0]);
 #pragma unroll
-                        for (int h = 0; h < CW / 16; ++h) {          // 16 columns at a time
-                            uint32_t r[16];
-                            ptx::tmem_ld_x16(taddr + (uint32_t)(16 * h), r);
-                            ptx::tmem_ld_wait();
+                        for (int h = 0; h < CW / 16; ++h) {          // 16 columns at a time, the next 16 on their way
+                            uint32_t (&r)[16] = rr[h & 1];
+                            ptx::tmem_ld_wait(r);
+                            if (h + 1 < CW / 16) ptx::tmem_ld_x16(taddr + (uint32_t)(16 * (h + 1)), rr[(h + 1) & 1]);
                             if constexpr (DUMP) {
                                 if (row_ok) {
 #pragma unroll
@@ -464,49 +465,52 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                     ptx::tc_fence_before();
                 }
                 __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&sh->slot_free[slot]));
+                if (ptx::elect_one()) ptx::mbar_arrive(ptx::smem_u32(&sh->slot_free[slot]));
                 if (++slot == NSLOT) { slot = 0; sphase ^= 1u; }
             }
 
-            if constexpr (!DUMP) {
+            if constexpr (!DUMP && SWAP) {
                 if (ok && active && row_ok) {
-                    if constexpr (SWAP) {
-                        // row = output channel, columns = tiles: contiguous in Y[p][k][:];
-                        // 32-byte stores so that every instruction fills whole sectors
-                        float *dst = a.Y + ((size_t)p * g.K + row) * g.Tp + col0;
+                    // row = output channel, columns = tiles: contiguous in Y[p][k][:];
+                    // 32-byte stores so that every instruction fills whole sectors
+                    float *dst = a.Y + ((size_t)p * g.K + row) * g.Tp + col0;
 #pragma unroll
-                        for (int j8 = 0; j8 < CW / 8; ++j8)
-                            if (col0 + 8 * j8 + 7 < g.Tp)
-                                ptx::st_global_v8(dst + 8 * j8, acc[4 * j8].x, acc[4 * j8].y, acc[4 * j8 + 1].x,
-                                                  acc[4 * j8 + 1].y, acc[4 * j8 + 2].x, acc[4 * j8 + 2].y,
-                                                  acc[4 * j8 + 3].x, acc[4 * j8 + 3].y);
-                    } else {
-                        // row = tile: lanes write consecutive t of one Y[p][k][:] row.  Whole blocks without
-                        // a test per column, the address advanced by the row pitch (forward, F(4,3), 784 tiles x
-                        // 320 channels 34.4 -> 33.6 us, F(6,3), 1600 x 320 78.4 -> 76.8 us).  A last block of
-                        // fewer columns ends at the first group of eight without one, which the tests of every
-                        // column did not (1600 tiles x 8 channels 23.1 -> 21.4 us, x 40 24.9 -> 24.0 us, x 136
-                        // 40.4 -> 39.3 us; with tests alone it was slower than before the whole blocks had
-                        // their own loop, 22.5 us for 8 channels)
-                        float *dst = a.Y + ((size_t)p * g.K + col0) * g.Tp + row;
-                        if (col0 + CW <= a.cols) {
+                    for (int j8 = 0; j8 < CW / 8; ++j8)
+                        if (col0 + 8 * j8 + 7 < g.Tp)
+                            ptx::st_global_v8(dst + 8 * j8, acc[4 * j8].x, acc[4 * j8].y, acc[4 * j8 + 1].x,
+                                              acc[4 * j8 + 1].y, acc[4 * j8 + 2].x, acc[4 * j8 + 2].y,
+                                              acc[4 * j8 + 3].x, acc[4 * j8 + 3].y);
+                }
+            } else if constexpr (!DUMP) {
+                if (ok && active) {
+                    // row = tile: the warp's columns go to shared memory as rows of 32 tiles and from there to
+                    // Y[p][k][t] by one tiled store, which leaves out what lies beyond K or T (rounded up to
+                    // 16 bytes, inside the padding of the row), while the warp goes
+                    // on with the next unit.  Stored by the warp itself (64 stores of 128 bytes) they held it up for
+                    // as long as L2 took them (about 1400 cycles a unit): forward, 1024 tiles x 256 channels in groups
+                    // of 32 43.1 -> 42.6 us, F(6,3) 968 tiles x 512 channels, two layers, 57.0 -> 55.5 us
+                    unsigned char *out = store + quarter * (C::STORE_BYTES / NUM_EPI_WARPS);
+                    float *out_lane = reinterpret_cast<float *>(out) + lane;
+                    if (lane == 0) ptx::bulk_wait_read();
+                    __syncwarp();
 #pragma unroll
-                            for (int j = 0; j < CW / 2; ++j) {
-                                dst[0] = acc[j].x;
-                                dst[g.Tp] = acc[j].y;
-                                dst += 2 * g.Tp;
-                            }
-                        } else {
-#pragma unroll
-                            for (int j = 0; j < CW / 2; ++j) {
-                                if (j % 4 == 0 && col0 + 2 * j >= a.cols) break;
-                                if (col0 + 2 * j < a.cols) dst[(size_t)(2 * j) * g.Tp] = acc[j].x;
-                                if (col0 + 2 * j + 1 < a.cols) dst[(size_t)(2 * j + 1) * g.Tp] = acc[j].y;
-                            }
-                        }
+                    for (int j = 0; j < CW / 2; ++j) {
+                        out_lane[(2 * j) * 32] = acc[j].x;
+                        out_lane[(2 * j + 1) * 32] = acc[j].y;
                     }
+                    ptx::fence_proxy_async_smem();
+                    __syncwarp();
+                    if (lane == 0) {
+                        ptx::tma_store_3d(&tmY, ptx::smem_u32(out), mt * BM + quarter * 32, col0, p);
+                        ptx::bulk_commit();
+                    }
+                    __syncwarp();
                 }
             }
+        }
+        if constexpr (!DUMP && !SWAP) {
+            if (lane == 0) ptx::bulk_wait();
+            __syncwarp();
         }
     }
 
@@ -521,7 +525,7 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
 template <int BN, bool SWAP, bool DUMP>
 cudaError_t launch_variant(const wfq_plan &plan, int32_t *acc_dump, cudaStream_t stream, bool pdl)
 {
-    using C = Cfg<BN>;
+    using C = Cfg<BN, SWAP>;
     const Geometry &g = plan.geo;
     GemmArgs a;
     a.row_scale = SWAP ? plan.sW : plan.ws.sX;
@@ -558,7 +562,7 @@ cudaError_t launch_variant(const wfq_plan &plan, int32_t *acc_dump, cudaStream_t
     cfg.numAttrs = pdl ? 1 : 0;
     const CUtensorMap &tmA = SWAP ? plan.tmap_wq : plan.tmap_xq;
     const CUtensorMap &tmB = SWAP ? plan.tmap_xq : plan.tmap_wq;
-    return cudaLaunchKernelEx(&cfg, kern, tmA, tmB, a, g);
+    return cudaLaunchKernelEx(&cfg, kern, tmA, tmB, plan.tmap_y, a, g);
 }
 
 // ---- tensor-pipe rate of tcgen05.mma kind::i8 -----------------------------------------
@@ -630,7 +634,7 @@ template <int BN, bool SWAP, bool DUMP>
 cudaError_t setup_variant()
 {
     return cudaFuncSetAttribute(gemm_dequant_kernel<BN, SWAP, DUMP>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<BN>::SMEM_BYTES);
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<BN, SWAP>::SMEM_BYTES);
 }
 
 }  // namespace

@@ -21,7 +21,6 @@ enum WaitId : int {
     kWaitTmemFull = 4,    // epilogue waiting for a finished accumulator
     kWaitDrain = 5,       // teardown waiting for copies in flight
     kWaitScaleEmpty = 6,  // scale loader waiting for a free ring slot
-    kWaitScaleFull = 7,   // epilogue waiting for a group's scales
     kWaitStripEmpty = 8,  // input transform: TMA producer waiting for a free strip buffer
     kWaitStripFull = 9,   // input transform: im2col warps waiting for a strip
     kWaitPairEmpty = 10,  // input transform: im2col warps waiting for a free operand tile
@@ -143,6 +142,7 @@ struct wfq_plan {
                                // 3 cp.async without 16-byte copies
 
     CUtensorMap tmap_xq;       // Xq as (C, T, P) bytes, 128B-swizzled boxes
+    CUtensorMap tmap_y;        // Y as (T, K, P), boxes of one epilogue warp of the contraction
     CUtensorMap tmap_wq;       // Wq as (C, K, P)
     bool tmap_xq_ok = false, tmap_wq_ok = false;
     bool gemm_swap = false;    // contraction rows are output channels instead of tiles
@@ -203,6 +203,7 @@ cudaError_t launch_mma_peak(const wfq_plan &plan, int n_cols, int mmas, cudaStre
 // (128, box_rows, 1) box and 128-byte swizzle.  Returns false on failure.
 bool encode_tmap_bytes3d(CUtensorMap *map, const void *base, int inner, int rows, int planes,
                          int box_rows);
+bool encode_tmap_y(wfq_plan &plan);   // plan.tmap_y for the plan's workspace and column block
 
 
 // CTAs of `threads` threads and `smem` bytes of dynamic shared memory that fit on one SM of

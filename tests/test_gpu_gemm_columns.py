@@ -1,6 +1,5 @@
-"""Output channel counts around the blocks of 64 columns of the contraction and the groups of eight in which a
-partial block is stored: the first K channels of a wider layer give the same values bit for bit, and nothing is
-written beyond them."""
+"""Edges of the contraction's units.  Output channel counts around the blocks of 64 columns: the first K channels of a
+wider layer give the same values bit for bit, and nothing is written beyond them."""
 import pytest
 
 from paper_2412_19867_b200 import binding as b
@@ -31,3 +30,32 @@ def test_partial_column_blocks(m, gs, bn):
         assert torch.equal(Y[:, :, :conv.T], want[:, :K]), K
         conv.check_status()
         conv.close()
+
+
+@pytest.mark.parametrize("T", [1, 31, 32, 33, 96, 127, 128, 129, 161, 257])
+def test_partial_row_blocks(T):
+    """Tile counts around the 32 tiles of a store and the 128 of a unit, rows = tiles (stored by TMA) and rows = channels
+    (stored by the lanes): within the rounding of the fp32 sums of the scaled group sums in 64 bits, and rows = tiles
+    writes nothing behind the 16 bytes of the last tile (the unit of a TMA store; rows of Y are padded to 32 tiles)."""
+    import torch
+    m, C, K, gs = 4, 192, 72, 64
+    gen = torch.Generator(device="cuda").manual_seed(T)
+    x = torch.randn((1, C, m, m * T), generator=gen, device="cuda").half()
+    conv = b.Conv(1, C, K, m, m * T, m, gs, "f16")
+    conv.prepare(torch.randn((K, C, 3, 3), generator=gen, device="cuda"))
+    assert conv.T == T
+    b.wfq_input_transform_quantize(conv.plan, x.data_ptr(), conv._stream())
+    xq, wq = conv.buffer(b.WFQ_BUF_XQ).double(), conv.buffer(b.WFQ_BUF_WQ).double()
+    sx, sw = conv.buffer(b.WFQ_BUF_SX).double(), conv.buffer(b.WFQ_BUF_SW).double()
+    terms = torch.stack([wq[:, :, g * gs:(g + 1) * gs] @ xq[:, :, g * gs:(g + 1) * gs].transpose(1, 2) *
+                         sw[:, g, :K, None] * sx[:, g, None, :T] for g in range(C // gs)])
+    # a product with each scale and a sum: each rounds once per group
+    bound = (C // gs + 2) * 2.0 ** -24 * terms.abs().sum(0)
+    for shape in (264, 164, 116):
+        b.wfq_plan_set_debug_option(conv.plan, b.WFQ_DEBUG_GEMM_SHAPE, shape)
+        Y = conv.buffer(b.WFQ_BUF_Y).fill_(float("nan"))
+        b.wfq_gemm_dequantize(conv.plan, conv._stream())
+        assert ((Y[:, :, :T].double() - terms.sum(0)).abs() <= bound).all(), shape
+        assert shape == 264 or torch.isnan(Y[:, :, (T + 3) // 4 * 4:]).all()
+    conv.check_status()
+    conv.close()
