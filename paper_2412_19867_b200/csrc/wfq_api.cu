@@ -132,16 +132,6 @@ bool encode_tmap_bytes3d(CUtensorMap *map, const void *base, int inner, int rows
                        CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
-bool encode_tmap_y(wfq_plan &plan)
-{
-    const Geometry &g = plan.geo;
-    const unsigned long long dims[3] = {(unsigned long long)g.T, (unsigned long long)g.K, (unsigned long long)g.P};
-    const unsigned long long strides[2] = {(unsigned long long)g.Tp * 4, (unsigned long long)g.K * g.Tp * 4};
-    const unsigned box[3] = {32u, (unsigned)plan.gemm_bn, 1u};
-    return encode_tmap(&plan.tmap_y, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, plan.ws.Y, dims, strides, box,
-                       CU_TENSOR_MAP_SWIZZLE_NONE);
-}
-
 }  // namespace wfq
 
 extern "C" {
@@ -306,7 +296,7 @@ wfq_status_t wfq_plan_set_workspace(wfq_plan_t *plan, void *dev_ptr, size_t byte
     const wfq::Geometry &g = plan->geo;
     plan->tmap_xq_ok = wfq::encode_tmap_bytes3d(&plan->tmap_xq, ws.Xq, g.C, g.T, g.P,
                                                plan->gemm_swap ? plan->gemm_bn : wfq::gemm_block_m());
-    if (!plan->tmap_xq_ok || !wfq::encode_tmap_y(*plan)) return WFQ_ERR_CUDA;
+    if (!plan->tmap_xq_ok || !wfq::plan_gemm_units(*plan)) return WFQ_ERR_CUDA;
     plan->has_workspace = true;
     return WFQ_OK;
 }
@@ -724,7 +714,7 @@ wfq_status_t wfq_plan_set_debug_option(wfq_plan_t *plan, wfq_debug_option_t opti
             if (plan->has_workspace)
                 plan->tmap_xq_ok = wfq::encode_tmap_bytes3d(&plan->tmap_xq, plan->ws.Xq, g.C, g.T, g.P,
                                                            swap ? bn : wfq::gemm_block_m()) &&
-                                   wfq::encode_tmap_y(*plan);
+                                   wfq::plan_gemm_units(*plan);
             if (plan->Wq)
                 plan->tmap_wq_ok = wfq::encode_tmap_bytes3d(&plan->tmap_wq, plan->Wq, g.C, g.K, g.P,
                                                            swap ? wfq::gemm_block_m() : bn);

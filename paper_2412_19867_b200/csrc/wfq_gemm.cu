@@ -50,6 +50,9 @@ constexpr int NUM_EPI_WARPS = 4;   // one per 32 TMEM lanes
 constexpr int FIRST_EPI_WARP = 4;
 constexpr int NUM_THREADS = 32 * (FIRST_EPI_WARP + NUM_EPI_WARPS);
 
+// Pieces of 16 columns in a part of a cut unit: halves of 64 and of 32 columns, thirds of 48.
+__host__ __device__ constexpr int part_pieces(int bn) { return bn == 64 ? 2 : 1; }
+
 struct Shared {
     uint64_t full[NSTAGES];     // operands of a stage have landed
     uint64_t empty[NSTAGES];    // the MMAs reading a stage have completed
@@ -59,8 +62,8 @@ struct Shared {
     volatile int abort;
 };
 
-// Normal orientation: the epilogue hands Y to the TMA unit through shared memory.  Three stages leave the room for it and
-// are no slower than four (forward, ten layers within 0.2 %; swapped, 36 tiles x 1280 channels F(6,3) 44.0 -> 43.6 us).
+// Normal orientation: the epilogue hands Y to the TMA unit through shared memory.  Three stages leave the room for it
+// and are no slower than four (forward, ten layers within 0.2 %; swapped, 36 tiles x 1280 channels F(6,3) 44.0 -> 43.6 us).
 template <int BN, bool SWAP>
 struct Cfg {
     static constexpr int STORE_BYTES = SWAP ? 0 : BM * BN * 4;
@@ -69,7 +72,6 @@ struct Cfg {
     static constexpr int CG_MAX = SLOT_COLS / BN;             // groups per chunk at most
     static constexpr int GROUP_SCALE_FLOATS = BM + BN;        // row scales, then column scales
     static constexpr int SLOT_SCALE_FLOATS = CG_MAX * GROUP_SCALE_FLOATS;
-    static constexpr int CW = BN;                             // columns per epilogue warp
     static constexpr size_t SMEM_BYTES = 1024 /*alignment slack*/ + (size_t)NSTAGES * STAGE_BYTES + STORE_BYTES +
                                          (size_t)NSLOT * SLOT_SCALE_FLOATS * sizeof(float) + sizeof(Shared);
 };
@@ -80,6 +82,8 @@ struct GemmArgs {
     int row_pitch, col_pitch;
     int rows, cols;           // valid rows / columns: (T, K) normal, (K, T) swapped
     int cg;                   // groups per chunk
+    int items;                // work items: whole units, then the parts of the units that are cut (plan_gemm_units)
+    int whole, parts;         // whole units, parts of a cut one
     float *Y;                 // [P][K][Tp]
     int32_t *acc_dump;        // [P][T][K][G] or null
     int *status;
@@ -88,34 +92,55 @@ struct GemmArgs {
     long long l2_prefetch_bytes;   // per CTA: filter bytes it may ask into L2 ahead of the previous kernel's end
 };
 
+// A work item: a unit, or a part of it: `np` pieces of 16 columns from piece p0 on.
+struct Item { int p, mt, nt, p0, np; };
+template <int BN, bool CUT>
+__device__ __forceinline__ Item item_of(const GemmArgs &a, int i, int MT, int NT)
+{
+    Item it;
+    it.p0 = 0;
+    it.np = BN / 16;
+    if (CUT && i >= a.whole) {
+        const int r = i - a.whole;
+        i = a.whole + r / a.parts;
+        it.p0 = r % a.parts * part_pieces(BN);
+        it.np = part_pieces(BN);
+    }
+    it.nt = i % NT;
+    it.mt = (i / NT) % MT;
+    it.p = i / (NT * MT);
+    return it;
+}
+
 // MMA issue loop for the common shapes in which the chunks tile a stage exactly
 // (GSTEPS MMAs per group, CGT groups per chunk, GSTEPS * CGT in {2, 4} MMAs per chunk):
 // per chunk one slot wait, the chunk's MMAs as straight-line code with constant
 // descriptor offsets and accumulate flags, one commit.  The generic loop in the kernel
 // spends several hundred cycles per MMA on its bookkeeping, which made the issuing
 // warp the bottleneck of every layer with more than one chunk per unit.
-template <int BN, bool SWAP, int GSTEPS, int CGT>
+template <int BN, bool SWAP, bool CUT, int GSTEPS, int CGT>
 __device__ __forceinline__ void mma_issue_aligned(Shared *sh, uint32_t tiles_lo, uint32_t tmem_base,
-                                                  int units, int KB, int last_slices, int lane,
-                                                  const WaitCtx &ctx)
+                                                  const GemmArgs &args, int MT, int NT, int KB,
+                                                  int last_slices, const WaitCtx &ctx)
 {
     using C = Cfg<BN, SWAP>;
     constexpr int CHUNK_STEPS = GSTEPS * CGT;            // MMAs per chunk
     constexpr int NCH = (BK / UK) / CHUNK_STEPS;         // chunks per stage
     static_assert(NCH >= 1 && NCH * CHUNK_STEPS == BK / UK, "chunks must tile a stage");
-    constexpr uint32_t idesc = ptx::idesc_i8(BM, BN);
     constexpr uint32_t dhi = ptx::smem_desc_sw128_hi();
     const uint32_t full0 = ptx::smem_u32(&sh->full[0]), empty0 = ptx::smem_u32(&sh->empty[0]);
     const uint32_t acc0 = ptx::smem_u32(&sh->acc_full[0]), free0 = ptx::smem_u32(&sh->slot_free[0]);
     int stage = 0, slot = 0;
     uint32_t phase = 0, sphase = 0;
-    for (int u = blockIdx.x; u < units; u += gridDim.x) {
+    for (int i = blockIdx.x; i < args.items; i += gridDim.x) {
+        const Item it = item_of<BN, CUT>(args, i, MT, NT);
+        const uint32_t idesc = ptx::idesc_i8(BM, 16 * it.np);
         for (int kb = 0; kb < KB; ++kb) {
             const int nslice = kb == KB - 1 ? last_slices : BK / UK;
             if (!__all_sync(0xffffffffu, wait_bounded(full0 + 8u * stage, phase, ctx, kWaitSmemFull)))
                 return;
             const uint32_t a_lo = tiles_lo + (uint32_t)(stage * (C::STAGE_BYTES >> 4));
-            const uint32_t b_lo = a_lo + (uint32_t)(A_BYTES >> 4);
+            const uint32_t b_lo = a_lo + (uint32_t)(A_BYTES >> 4) + (uint32_t)(it.p0 * (16 * BK >> 4));
 #pragma unroll
             for (int c = 0; c < NCH; ++c) {
                 if (c * CHUNK_STEPS < nslice) {           // the chunk has at least one group
@@ -156,13 +181,136 @@ __device__ __forceinline__ void mma_issue_aligned(Shared *sh, uint32_t tiles_lo,
     }
 }
 
-template <int BN, bool SWAP, bool DUMP>
+// What the epilogue keeps through the kernel: the warp's tensor memory, the scale slots, its part of the staging for Y.
+struct EpiCtx {
+    uint32_t tmem;
+    const float *scales;
+    unsigned char *out;
+    int quarter, lane, nchunk;
+};
+
+// One work item in the epilogue: NP * 16 columns from column block0 + c0 on, c0 inside the unit's block of BN columns.
+template <int BN, bool SWAP, bool DUMP, bool CUT, int NP>
+__device__ __forceinline__ bool epilogue_unit(Shared *sh, const CUtensorMap &tmY, const GemmArgs &a, const Geometry &g,
+                                              const WaitCtx &ctx, const EpiCtx &ec, int p, int mt, int block0, int c0,
+                                              int &slot, uint32_t &sphase)
+{
+    using C = Cfg<BN, SWAP>;
+    constexpr int CW = 16 * NP;                                // columns of the item
+    constexpr int SW = CUT ? 16 * part_pieces(BN) : BN;        // columns of a store (a box of tmap_y)
+    const int quarter = ec.quarter, lane = ec.lane;
+    const int row = mt * BM + quarter * 32 + lane;    // tile (normal) or channel (swapped)
+    const int col0 = block0 + c0;                     // first column
+    // warp-uniform: does this warp own any valid row and column of the unit?
+    const bool active = (mt * BM + quarter * 32 < a.rows) && (col0 < a.cols);
+    const bool row_ok = row < a.rows;
+    float2 acc[CW / 2];
+#pragma unroll
+    for (int j = 0; j < CW / 2; ++j) acc[j] = make_float2(0.f, 0.f);
+
+    for (int ch = 0; ch < ec.nchunk; ++ch) {
+        const int g0 = ch * a.cg, ng = min(a.cg, g.G - g0);
+        if (!wait_bounded(ptx::smem_u32(&sh->acc_full[slot]), sphase, ctx, kWaitTmemFull)) return false;
+        if (active) {
+            ptx::tc_fence_after();
+            const float *sc = ec.scales + (size_t)slot * C::SLOT_SCALE_FLOATS;
+            for (int j = 0; j < ng; ++j) {
+                const uint32_t taddr = ec.tmem + (uint32_t)(slot * SLOT_COLS + j * BN);
+                const float rs = sc[j * C::GROUP_SCALE_FLOATS + quarter * 32 + lane];
+                const float2 rs2 = make_float2(rs, rs);
+                const float4 *cs4 = reinterpret_cast<const float4 *>(sc + j * C::GROUP_SCALE_FLOATS + BM + c0);
+                uint32_t rr[2][16];
+                ptx::tmem_ld_x16(taddr, rr[0]);
+#pragma unroll
+                for (int h = 0; h < CW / 16; ++h) {          // 16 columns at a time, the next 16 on their way
+                    uint32_t (&r)[16] = rr[h & 1];
+                    ptx::tmem_ld_wait(r);
+                    if (h + 1 < CW / 16) ptx::tmem_ld_x16(taddr + (uint32_t)(16 * (h + 1)), rr[(h + 1) & 1]);
+                    if constexpr (DUMP) {
+                        if (row_ok) {
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) {
+                                const int col = col0 + 16 * h + i;
+                                if (col < a.cols) {
+                                    const size_t t = SWAP ? col : row, k = SWAP ? row : col;
+                                    a.acc_dump[(((size_t)p * g.T + t) * g.K + k) * g.G + g0 + j] =
+                                        (int32_t)r[i];
+                                }
+                            }
+                        }
+                    } else {
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const float4 cs = cs4[4 * h + q];
+                            float2 f0 = make_float2(__int2float_rn((int32_t)r[4 * q + 0]),
+                                                    __int2float_rn((int32_t)r[4 * q + 1]));
+                            float2 f1 = make_float2(__int2float_rn((int32_t)r[4 * q + 2]),
+                                                    __int2float_rn((int32_t)r[4 * q + 3]));
+                            f0 = __fmul2_rn(f0, rs2);
+                            f1 = __fmul2_rn(f1, rs2);
+                            acc[8 * h + 2 * q] = __ffma2_rn(f0, make_float2(cs.x, cs.y), acc[8 * h + 2 * q]);
+                            acc[8 * h + 2 * q + 1] =
+                                __ffma2_rn(f1, make_float2(cs.z, cs.w), acc[8 * h + 2 * q + 1]);
+                        }
+                    }
+                }
+            }
+            ptx::tc_fence_before();
+        }
+        __syncwarp();
+        if (ptx::elect_one()) ptx::mbar_arrive(ptx::smem_u32(&sh->slot_free[slot]));
+        if (++slot == NSLOT) { slot = 0; sphase ^= 1u; }
+    }
+
+    if constexpr (!DUMP && SWAP) {
+        if (active && row_ok) {
+            // row = output channel, columns = tiles: contiguous in Y[p][k][:];
+            // 32-byte stores so that every instruction fills whole sectors
+            float *dst = a.Y + ((size_t)p * g.K + row) * g.Tp + col0;
+#pragma unroll
+            for (int j8 = 0; j8 < CW / 8; ++j8)
+                if (col0 + 8 * j8 + 7 < g.Tp)
+                    ptx::st_global_v8(dst + 8 * j8, acc[4 * j8].x, acc[4 * j8].y, acc[4 * j8 + 1].x,
+                                      acc[4 * j8 + 1].y, acc[4 * j8 + 2].x, acc[4 * j8 + 2].y,
+                                      acc[4 * j8 + 3].x, acc[4 * j8 + 3].y);
+        }
+    } else if constexpr (!DUMP) {
+        if (active) {
+            // row = tile: the warp's columns go to shared memory as rows of 32 tiles and from there to Y[p][k][t] by
+            // tiled stores, which leave out what lies beyond K or T (rounded up to 16 bytes, inside the padding of the
+            // row), while the warp goes on with the next item.  Stored by the warp itself (64 stores of 128 bytes) they
+            // held it up for as long as L2 took them (about 1400 cycles a unit): forward, 1024 tiles x 256 channels in
+            // groups of 32 43.1 -> 42.6 us, F(6,3) 128 tiles x 512 channels, two layers, 57.0 -> 55.5 us
+            float *out_lane = reinterpret_cast<float *>(ec.out) + lane;
+            if (lane == 0) ptx::bulk_wait_read();
+            __syncwarp();
+#pragma unroll
+            for (int j = 0; j < CW / 2; ++j) {
+                out_lane[(2 * j) * 32] = acc[j].x;
+                out_lane[(2 * j + 1) * 32] = acc[j].y;
+            }
+            ptx::fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+#pragma unroll
+                for (int h = 0; h < CW; h += SW)
+                    if (col0 + h < a.cols)
+                        ptx::tma_store_3d(&tmY, ptx::smem_u32(ec.out) + (uint32_t)(h * 128), mt * BM + quarter * 32,
+                                          col0 + h, p);
+                ptx::bulk_commit();
+            }
+            __syncwarp();
+        }
+    }
+    return true;
+}
+
+template <int BN, bool SWAP, bool DUMP, bool CUT>
 __global__ void __launch_bounds__(NUM_THREADS, 2)
 gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                     const __grid_constant__ CUtensorMap tmY, GemmArgs a, Geometry g)
 {
     using C = Cfg<BN, SWAP>;
-    constexpr int CW = C::CW;
     extern __shared__ unsigned char smem_raw[];
     // 1024-byte alignment: the 128-byte swizzle atoms repeat every 1024 bytes
     unsigned char *tiles = ptx::align_smem<1024>(smem_raw);
@@ -172,7 +320,6 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int MT = (a.rows + BM - 1) / BM, NT = (a.cols + BN - 1) / BN;
-    const int units = g.P * MT * NT;
     const int KB = (g.C + BK - 1) / BK;          // stages per unit
     const int gs_steps = g.gs / UK;              // MMAs per group
     const int cg = a.cg;                         // groups per chunk
@@ -208,16 +355,16 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     // wait for it.
     constexpr int W_ROWS = SWAP ? BM : BN;                 // filter rows of a stage
     // stages of the first unit whose filter half is loaded early
-    const int pre = (a.l2_prefetch_bytes > 0 && (int)blockIdx.x < units) ? (KB < NSTAGES ? KB : NSTAGES) : 0;
+    const int pre = (a.l2_prefetch_bytes > 0 && (int)blockIdx.x < a.items) ? (KB < NSTAGES ? KB : NSTAGES) : 0;
     if (warp == 0 && ptx::elect_one()) {
         ptx::prefetch_tmap(&tmA);
         ptx::prefetch_tmap(&tmB);
         if (!SWAP) ptx::prefetch_tmap(&tmY);
         const CUtensorMap *tmW = SWAP ? &tmA : &tmB;
         long long budget = a.l2_prefetch_bytes;
-        for (int u = blockIdx.x, first = 1; u < units && budget > 0; u += gridDim.x, first = 0) {
-            const int nt = u % NT, mt = (u / NT) % MT, p = u / (NT * MT);
-            const int wrow = SWAP ? mt * BM : nt * BN;
+        for (int i = blockIdx.x, first = 1; i < a.items && budget > 0; i += gridDim.x, first = 0) {
+            const Item it = item_of<BN, CUT>(a, i, MT, NT);
+            const int p = it.p, wrow = SWAP ? it.mt * BM : it.nt * BN;
             for (int kb = 0; kb < KB && budget > 0; ++kb) {
                 if (first && kb < pre) {
                     if (!(blockIdx.x == 0 && kb == a.debug_skip_stage)) {
@@ -245,8 +392,9 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         uint32_t phase = 0;
         long long issued = 0;
         bool ok = true;
-        for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
-            const int nt = u % NT, mt = (u / NT) % MT, p = u / (NT * MT);
+        for (int i = blockIdx.x; i < a.items && ok; i += gridDim.x) {
+            const Item it = item_of<BN, CUT>(a, i, MT, NT);
+            const int nt = it.nt, mt = it.mt, p = it.p;
             for (int kb = 0; kb < KB; ++kb) {
                 ok = __all_sync(0xffffffffu, wait_bounded(ptx::smem_u32(&sh->empty[stage]), phase ^ 1u, ctx,
                                                           kWaitSmemEmpty));
@@ -284,7 +432,6 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         // The warp stays converged; lane 0 issues every MMA and commit.  Its instructions
         // form one dependent chain, so the descriptors are advanced with 32-bit adds and
         // the accumulate flag is a constant of the instruction.
-        constexpr uint32_t idesc = ptx::idesc_i8(BM, BN);
         constexpr uint32_t dhi = ptx::smem_desc_sw128_hi();
         const uint32_t tiles_lo = ptx::smem_desc_sw128_lo(ptx::smem_u32(tiles));
         const int chunk_steps = cg * gs_steps;       // MMAs per full chunk
@@ -294,17 +441,19 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         bool ok = true;
         // shapes whose chunks tile a stage exactly take the straight-line issue loop
         if (gs_steps == 2 && cg == 2) {
-            mma_issue_aligned<BN, SWAP, 2, 2>(sh, tiles_lo, tmem_base, units, KB, last_slices, lane, ctx);
+            mma_issue_aligned<BN, SWAP, CUT, 2, 2>(sh, tiles_lo, tmem_base, a, MT, NT, KB, last_slices, ctx);
             ok = false;
         } else if (gs_steps == 4 && cg == 1) {
-            mma_issue_aligned<BN, SWAP, 4, 1>(sh, tiles_lo, tmem_base, units, KB, last_slices, lane, ctx);
+            mma_issue_aligned<BN, SWAP, CUT, 4, 1>(sh, tiles_lo, tmem_base, a, MT, NT, KB, last_slices, ctx);
             ok = false;
         } else if (gs_steps == 1 && cg == C::CG_MAX && C::CG_MAX <= 4) {
-            mma_issue_aligned<BN, SWAP, 1, (C::CG_MAX <= 4 ? C::CG_MAX : 4)>(sh, tiles_lo, tmem_base, units, KB,
-                                                                    last_slices, lane, ctx);
+            mma_issue_aligned<BN, SWAP, CUT, 1, (C::CG_MAX <= 4 ? C::CG_MAX : 4)>(sh, tiles_lo, tmem_base, a, MT, NT,
+                                                                                  KB, last_slices, ctx);
             ok = false;
         }
-        for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+        for (int i = blockIdx.x; i < a.items && ok; i += gridDim.x) {
+            const Item it = item_of<BN, CUT>(a, i, MT, NT);
+            const uint32_t idesc = ptx::idesc_i8(BM, 16 * it.np);
             int step = 0;          // MMA step within the chunk
             int in_group = 0;      // MMA step within the group
             uint32_t dcol = 0;     // TMEM column of the current group
@@ -315,7 +464,7 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 ptx::tc_fence_after();
                 // a 32-byte step along K inside the swizzled rows is +2 in the address field
                 const uint32_t a_lo = tiles_lo + (uint32_t)(stage * (C::STAGE_BYTES >> 4));
-                const uint32_t b_lo = a_lo + (uint32_t)(A_BYTES >> 4);
+                const uint32_t b_lo = a_lo + (uint32_t)(A_BYTES >> 4) + (uint32_t)(it.p0 * (16 * BK >> 4));
                 const int nslice = min(BK, g.C - kb * BK) / UK;
                 for (int s = 0; s < nslice; ++s) {
                     if (step == 0) {
@@ -357,8 +506,9 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             uint32_t sphase = 0;
             long long issued = 0;
             bool ok = true;
-            for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
-                const int nt = u % NT, mt = (u / NT) % MT, p = u / (NT * MT);
+            for (int i = blockIdx.x; i < a.items && ok; i += gridDim.x) {
+                const Item it = item_of<BN, CUT>(a, i, MT, NT);
+                const int nt = it.nt, mt = it.mt, p = it.p;
                 for (int ch = 0; ch < nchunk; ++ch) {
                     const int g0 = ch * cg, ng = min(cg, g.G - g0);
                     ok = __all_sync(0xffffffffu, wait_bounded(ptx::smem_u32(&sh->slot_free[slot]), sphase ^ 1u,
@@ -396,117 +546,22 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     } else if (warp >= FIRST_EPI_WARP) {
         // ---------------- epilogue ----------------
         const int quarter = warp & 3;                         // TMEM lanes this warp may read
-        const int c0 = ((warp - FIRST_EPI_WARP) >> 2) * CW;   // first column of this warp
-        const uint32_t tmem_warp = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c0;
         int slot = 0;
         uint32_t sphase = 0;
         bool ok = true;
-        for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
-            const int nt = u % NT, mt = (u / NT) % MT, p = u / (NT * MT);
-            const int row = mt * BM + quarter * 32 + lane;    // tile (normal) or channel (swapped)
-            const int col0 = nt * BN + c0;
-            // warp-uniform: does this warp own any valid row and column of the unit?
-            const bool active = (mt * BM + quarter * 32 < a.rows) && (col0 < a.cols);
-            const bool row_ok = row < a.rows;
-            float2 acc[CW / 2];
-#pragma unroll
-            for (int j = 0; j < CW / 2; ++j) acc[j] = make_float2(0.f, 0.f);
-
-            for (int ch = 0; ch < nchunk && ok; ++ch) {
-                const int g0 = ch * cg, ng = min(cg, g.G - g0);
-                if (!wait_bounded(ptx::smem_u32(&sh->acc_full[slot]), sphase, ctx, kWaitTmemFull)) {
-                    ok = false; break;
-                }
-                if (active) {
-                    ptx::tc_fence_after();
-                    const float *sc = scales + (size_t)slot * C::SLOT_SCALE_FLOATS;
-                    for (int j = 0; j < ng; ++j) {
-                        const uint32_t taddr = tmem_warp + (uint32_t)(slot * SLOT_COLS + j * BN);
-                        const float rs = sc[j * C::GROUP_SCALE_FLOATS + quarter * 32 + lane];
-                        const float2 rs2 = make_float2(rs, rs);
-                        const float4 *cs4 = reinterpret_cast<const float4 *>(
-                            sc + j * C::GROUP_SCALE_FLOATS + BM + c0);
-                        uint32_t rr[2][16];
-                        ptx::tmem_ld_x16(taddr, rr[0]);
-#pragma unroll
-                        for (int h = 0; h < CW / 16; ++h) {          // 16 columns at a time, the next 16 on their way
-                            uint32_t (&r)[16] = rr[h & 1];
-                            ptx::tmem_ld_wait(r);
-                            if (h + 1 < CW / 16) ptx::tmem_ld_x16(taddr + (uint32_t)(16 * (h + 1)), rr[(h + 1) & 1]);
-                            if constexpr (DUMP) {
-                                if (row_ok) {
-#pragma unroll
-                                    for (int i = 0; i < 16; ++i) {
-                                        const int col = col0 + 16 * h + i;
-                                        if (col < a.cols) {
-                                            const size_t t = SWAP ? col : row, k = SWAP ? row : col;
-                                            a.acc_dump[(((size_t)p * g.T + t) * g.K + k) * g.G + g0 + j] =
-                                                (int32_t)r[i];
-                                        }
-                                    }
-                                }
-                            } else {
-#pragma unroll
-                                for (int q = 0; q < 4; ++q) {
-                                    const float4 cs = cs4[4 * h + q];
-                                    float2 f0 = make_float2(__int2float_rn((int32_t)r[4 * q + 0]),
-                                                            __int2float_rn((int32_t)r[4 * q + 1]));
-                                    float2 f1 = make_float2(__int2float_rn((int32_t)r[4 * q + 2]),
-                                                            __int2float_rn((int32_t)r[4 * q + 3]));
-                                    f0 = __fmul2_rn(f0, rs2);
-                                    f1 = __fmul2_rn(f1, rs2);
-                                    acc[8 * h + 2 * q] = __ffma2_rn(f0, make_float2(cs.x, cs.y), acc[8 * h + 2 * q]);
-                                    acc[8 * h + 2 * q + 1] =
-                                        __ffma2_rn(f1, make_float2(cs.z, cs.w), acc[8 * h + 2 * q + 1]);
-                                }
-                            }
-                        }
-                    }
-                    ptx::tc_fence_before();
-                }
-                __syncwarp();
-                if (ptx::elect_one()) ptx::mbar_arrive(ptx::smem_u32(&sh->slot_free[slot]));
-                if (++slot == NSLOT) { slot = 0; sphase ^= 1u; }
-            }
-
-            if constexpr (!DUMP && SWAP) {
-                if (ok && active && row_ok) {
-                    // row = output channel, columns = tiles: contiguous in Y[p][k][:];
-                    // 32-byte stores so that every instruction fills whole sectors
-                    float *dst = a.Y + ((size_t)p * g.K + row) * g.Tp + col0;
-#pragma unroll
-                    for (int j8 = 0; j8 < CW / 8; ++j8)
-                        if (col0 + 8 * j8 + 7 < g.Tp)
-                            ptx::st_global_v8(dst + 8 * j8, acc[4 * j8].x, acc[4 * j8].y, acc[4 * j8 + 1].x,
-                                              acc[4 * j8 + 1].y, acc[4 * j8 + 2].x, acc[4 * j8 + 2].y,
-                                              acc[4 * j8 + 3].x, acc[4 * j8 + 3].y);
-                }
-            } else if constexpr (!DUMP) {
-                if (ok && active) {
-                    // row = tile: the warp's columns go to shared memory as rows of 32 tiles and from there to
-                    // Y[p][k][t] by one tiled store, which leaves out what lies beyond K or T (rounded up to
-                    // 16 bytes, inside the padding of the row), while the warp goes
-                    // on with the next unit.  Stored by the warp itself (64 stores of 128 bytes) they held it up for
-                    // as long as L2 took them (about 1400 cycles a unit): forward, 1024 tiles x 256 channels in groups
-                    // of 32 43.1 -> 42.6 us, F(6,3) 968 tiles x 512 channels, two layers, 57.0 -> 55.5 us
-                    unsigned char *out = store + quarter * (C::STORE_BYTES / NUM_EPI_WARPS);
-                    float *out_lane = reinterpret_cast<float *>(out) + lane;
-                    if (lane == 0) ptx::bulk_wait_read();
-                    __syncwarp();
-#pragma unroll
-                    for (int j = 0; j < CW / 2; ++j) {
-                        out_lane[(2 * j) * 32] = acc[j].x;
-                        out_lane[(2 * j + 1) * 32] = acc[j].y;
-                    }
-                    ptx::fence_proxy_async_smem();
-                    __syncwarp();
-                    if (lane == 0) {
-                        ptx::tma_store_3d(&tmY, ptx::smem_u32(out), mt * BM + quarter * 32, col0, p);
-                        ptx::bulk_commit();
-                    }
-                    __syncwarp();
-                }
-            }
+        const EpiCtx ec{tmem_base + ((uint32_t)(quarter * 32) << 16), scales,
+                        store + quarter * (C::STORE_BYTES / NUM_EPI_WARPS), quarter, lane, nchunk};
+        // The parts of cut units (at most one per CTA) run code of their own: a bound on the pieces inside the unrolled
+        // loops keeps the compiler from interleaving them (all layers 10 % slower)
+        for (int i = blockIdx.x; i < a.whole && ok; i += gridDim.x) {
+            const int nt = i % NT, mt = (i / NT) % MT, p = i / (NT * MT);
+            ok = epilogue_unit<BN, SWAP, DUMP, CUT, BN / 16>(sh, tmY, a, g, ctx, ec, p, mt, nt * BN, 0, slot, sphase);
+        }
+        const int tail = a.whole + (int)blockIdx.x;
+        if (CUT && tail < a.items && ok) {
+            const Item it = item_of<BN, CUT>(a, tail, MT, NT);
+            ok = epilogue_unit<BN, SWAP, DUMP, CUT, part_pieces(BN)>(sh, tmY, a, g, ctx, ec, it.p, it.mt, it.nt * BN,
+                                                                     16 * it.p0, slot, sphase);
         }
         if constexpr (!DUMP && !SWAP) {
             if (lane == 0) ptx::bulk_wait();
@@ -522,6 +577,14 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     }
 }
 
+// Groups per chunk: as many whole groups as fit into 128 channels (one stage) and into one TMEM slot; group sizes that
+// do not divide 128 get one group per chunk.
+int groups_per_chunk(int gs, int bn)
+{
+    if (BK % gs != 0) return 1;
+    return BK / gs < SLOT_COLS / bn ? BK / gs : SLOT_COLS / bn;
+}
+
 template <int BN, bool SWAP, bool DUMP>
 cudaError_t launch_variant(const wfq_plan &plan, int32_t *acc_dump, cudaStream_t stream, bool pdl)
 {
@@ -534,22 +597,24 @@ cudaError_t launch_variant(const wfq_plan &plan, int32_t *acc_dump, cudaStream_t
     a.col_pitch = SWAP ? g.Ts : g.Kp;
     a.rows = SWAP ? g.K : g.T;
     a.cols = SWAP ? g.T : g.K;
-    // groups per chunk: as many whole groups as fit into 128 channels (one stage) and
-    // into one TMEM slot; group sizes that do not divide 128 get one group per chunk
-    a.cg = 1;
-    if (BK % g.gs == 0) a.cg = BK / g.gs < C::CG_MAX ? BK / g.gs : C::CG_MAX;
+    a.cg = groups_per_chunk(g.gs, BN);
     a.Y = plan.ws.Y;
     a.acc_dump = acc_dump;
     a.status = plan.status;
     a.wait_cycles = plan.wait_cycles;
     a.debug_skip_stage = plan.debug_skip_gemm_stage;
     const int MT = (a.rows + BM - 1) / BM, NT = (a.cols + BN - 1) / BN;
-    const int units = g.P * MT * NT;
     const int slots = 2 * plan.sm_count;          // two CTAs per SM
-    const int grid = units < slots ? units : slots;
+    const int units = g.P * MT * NT;
+    a.whole = DUMP ? units : plan.gemm_whole;     // the debug output is not cut
+    a.parts = DUMP ? 1 : plan.gemm_parts;
+    a.items = a.whole + (units - a.whole) * a.parts;
+    const int grid = a.items < slots ? a.items : slots;
     // the filters share L2 (126 MB) with Xq, sX and Y: at most 48 MB of them are asked for early
     a.l2_prefetch_bytes = pdl ? (48LL << 20) / grid : 0;
-    auto kern = gemm_dequant_kernel<BN, SWAP, DUMP>;
+    auto kern = gemm_dequant_kernel<BN, SWAP, DUMP, false>;
+    if constexpr (BN != 16 && !DUMP)
+        if (a.parts > 1) kern = gemm_dequant_kernel<BN, SWAP, DUMP, true>;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3(NUM_THREADS);
@@ -633,7 +698,13 @@ cudaError_t launch_peak(int grid, int mmas, int *status, long long wait_cycles, 
 template <int BN, bool SWAP, bool DUMP>
 cudaError_t setup_variant()
 {
-    return cudaFuncSetAttribute(gemm_dequant_kernel<BN, SWAP, DUMP>,
+    if constexpr (BN != 16 && !DUMP) {
+        const cudaError_t e = cudaFuncSetAttribute(gemm_dequant_kernel<BN, SWAP, DUMP, true>,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)Cfg<BN, SWAP>::SMEM_BYTES);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaFuncSetAttribute(gemm_dequant_kernel<BN, SWAP, DUMP, false>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<BN, SWAP>::SMEM_BYTES);
 }
 
@@ -666,6 +737,31 @@ cudaError_t launch_mma_peak(const wfq_plan &plan, int n_cols, int mmas, cudaStre
         case 256: return launch_peak<256>(grid, mmas, plan.status, plan.wait_cycles, stream);
         default: return cudaErrorInvalidValue;
     }
+}
+
+// Which units are cut into parts along their columns, and the box of the stores of Y.  A last round that leaves CTAs
+// without a unit takes as long as a full one; where it holds no more units than parts of them have room, each CTA of
+// it takes a part (forward: 360 units of 5 chunks on 296 CTAs 33.4 -> 32.4 us, 640 units 35.8 -> 34.9 us, swapped in
+// thirds of 48 columns 43.6 -> 42.5 us, 54 units of 3 chunks 13.8 -> 12.8 us).  Units of one chunk are no shorter in
+// parts (84 of 972 units with 40 columns 23.9 -> 24.5 us), nor is a unit whose columns all lie in its first part.
+// Quarters of 64 columns, where they fit, are as good as halves (F(2,3) 1216 channels 78.9 -> 77.0 us, 640 units
+// 34.9 -> 35.4 us).
+bool plan_gemm_units(wfq_plan &plan)
+{
+    const Geometry &g = plan.geo;
+    const int bn = plan.gemm_bn, rows = plan.gemm_swap ? g.K : g.T, cols = plan.gemm_swap ? g.T : g.K;
+    const int units = g.P * ((rows + BM - 1) / BM) * ((cols + bn - 1) / bn), slots = 2 * plan.sm_count;
+    const int rest = slots > 0 ? units % slots : 0;
+    const int part = 16 * part_pieces(bn), parts = bn / part;
+    const int cg = groups_per_chunk(g.gs, bn);
+    const bool cut = parts > 1 && rest > 0 && parts * rest <= slots && (g.G + cg - 1) / cg > 1 && cols > part;
+    plan.gemm_whole = cut ? units - rest : units;
+    plan.gemm_parts = cut ? parts : 1;
+    const unsigned long long dims[3] = {(unsigned long long)g.T, (unsigned long long)g.K, (unsigned long long)g.P};
+    const unsigned long long strides[2] = {(unsigned long long)g.Tp * 4, (unsigned long long)g.K * g.Tp * 4};
+    const unsigned box[3] = {32u, (unsigned)(cut ? part : bn), 1u};
+    return encode_tmap(&plan.tmap_y, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, plan.ws.Y, dims, strides, box,
+                       CU_TENSOR_MAP_SWIZZLE_NONE);
 }
 
 int gemm_block_m() { return BM; }

@@ -142,11 +142,13 @@ struct wfq_plan {
                                // 3 cp.async without 16-byte copies
 
     CUtensorMap tmap_xq;       // Xq as (C, T, P) bytes, 128B-swizzled boxes
-    CUtensorMap tmap_y;        // Y as (T, K, P), boxes of one epilogue warp of the contraction
+    CUtensorMap tmap_y;        // Y as (T, K, P), boxes of one store of an epilogue warp of the contraction
     CUtensorMap tmap_wq;       // Wq as (C, K, P)
     bool tmap_xq_ok = false, tmap_wq_ok = false;
     bool gemm_swap = false;    // contraction rows are output channels instead of tiles
     int gemm_bn = 64;          // columns per unit of the contraction
+    int gemm_whole = 0;        // units of the contraction that are one work item each; the others are cut into
+    int gemm_parts = 1;        // this many parts along their columns
 
     // wfq_conv_forward_host on batches of several images: the batch is cut into chunks
     // of whole images that alternate between two internal streams, so that the copy in
@@ -203,7 +205,7 @@ cudaError_t launch_mma_peak(const wfq_plan &plan, int n_cols, int mmas, cudaStre
 // (128, box_rows, 1) box and 128-byte swizzle.  Returns false on failure.
 bool encode_tmap_bytes3d(CUtensorMap *map, const void *base, int inner, int rows, int planes,
                          int box_rows);
-bool encode_tmap_y(wfq_plan &plan);   // plan.tmap_y for the plan's workspace and column block
+bool plan_gemm_units(wfq_plan &plan);   // gemm_whole, gemm_parts and tmap_y for the plan's device, workspace and column block
 
 
 // CTAs of `threads` threads and `smem` bytes of dynamic shared memory that fit on one SM of

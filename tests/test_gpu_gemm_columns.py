@@ -51,11 +51,11 @@ def test_partial_row_blocks(T):
                          sw[:, g, :K, None] * sx[:, g, None, :T] for g in range(C // gs)])
     # a product with each scale and a sum: each rounds once per group
     bound = (C // gs + 2) * 2.0 ** -24 * terms.abs().sum(0)
-    for shape in (264, 164, 116):
+    for shape in (264, 248, 232, 164, 116):      # up to 128 tiles the units of 64, 48 and 32 columns are cut into parts
         b.wfq_plan_set_debug_option(conv.plan, b.WFQ_DEBUG_GEMM_SHAPE, shape)
         Y = conv.buffer(b.WFQ_BUF_Y).fill_(float("nan"))
         b.wfq_gemm_dequantize(conv.plan, conv._stream())
         assert ((Y[:, :, :T].double() - terms.sum(0)).abs() <= bound).all(), shape
-        assert shape == 264 or torch.isnan(Y[:, :, (T + 3) // 4 * 4:]).all()
+        assert shape >= 200 or torch.isnan(Y[:, :, (T + 3) // 4 * 4:]).all()
     conv.check_status()
     conv.close()
