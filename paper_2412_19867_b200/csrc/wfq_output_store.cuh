@@ -45,7 +45,9 @@ __device__ __forceinline__ void epilogue(float (&o)[M], float bias, int act)
 // kernel bound by them).  The CTA therefore collects its tiles' outputs in shared memory,
 // one array per output row u with the tiles side by side exactly as they lie in the image
 // row, and copies them out with consecutive lanes on consecutive 8 bytes (even W) or
-// consecutive floats (odd W).
+// consecutive floats (odd W).  A thread keeps its place in the rows and goes down them: tile, limits and offset are
+// formed once per place instead of once per element (most of the instructions of the copy; forward, 128 tiles x 512
+// channels of 7x7 images, two layers, 55.7 -> 53.1 us; ten 22x15 images, 64 channels, integer transforms 24.8 -> 23.6).
 // What one thread per tile of a CTA's TT (64 or 128) tiles has computed goes to y: `row_of(u, o)` gives row u of the
 // thread's tile (called once per u), base is the offset of y[img][k][h0][w0].
 template <int M, int STORE, int TT>
@@ -83,39 +85,42 @@ __device__ __forceinline__ void store_tiles(const RowOf &row_of, StoreShared<M, 
         tile_lim[j] = live ? (min(M, g.H - h0) * 16 + min(M, g.W - w0)) : 0;
         __syncthreads();
         if constexpr (STORE == 0) {
-            // float f of row u: tile f / M, column f % M
+            // float f of a row: tile f / M, column f % M
 #pragma unroll
-            for (int u = 0; u < M; ++u) {
-                const float *row = out_s + u * TT * M;
+            for (int i = 0; i < M; ++i) {
+                const int f = threadIdx.x + i * TT;
+                const int tj = f / M, v1 = f - tj * M;
+                const int lim = tile_lim[tj], rows = v1 < (lim & 15) ? lim >> 4 : 0;
+                size_t off = (size_t)tile_base[tj] + v1;
+                const float *src = out_s + f;
 #pragma unroll
-                for (int i = 0; i < M; ++i) {
-                    const int f = threadIdx.x + i * TT;
-                    const int tj = f / M, v1 = f - tj * M;
-                    const int lim = tile_lim[tj];
-                    if (u < (lim >> 4) && v1 < (lim & 15)) {
-                        const size_t off = (size_t)tile_base[tj] + (size_t)u * g.W + v1;
-                        if (EPI && out_half) yh[off] = to_bits16(row[f], out_half);
-                        else y[off] = row[f];
+                for (int u = 0; u < M; ++u) {
+                    if (u < rows) {
+                        if (EPI && out_half) yh[off] = to_bits16(src[u * TT * M], out_half);
+                        else y[off] = src[u * TT * M];
                     }
+                    off += g.W;
                 }
             }
             return;
         }
-        // pair q of row u: tile q / (M/2), columns 2 * (q % (M/2)) and the next
+        // pair q of a row: tile q / (M/2), columns 2 * (q % (M/2)) and the next
         constexpr int PPT = M / 2;                // pairs per tile row
 #pragma unroll
-        for (int u = 0; u < M; ++u) {
-            const float2 *row = reinterpret_cast<const float2 *>(out_s + u * TT * M);
+        for (int i = 0; i < PPT; ++i) {
+            const int q = threadIdx.x + i * TT;
+            const int tj = q / PPT, v2 = 2 * (q - tj * PPT);
+            const int lim = tile_lim[tj], rows = v2 < (lim & 15) ? lim >> 4 : 0;    // W even: both columns or none
+            size_t off = (size_t)tile_base[tj] + v2;
+            const float2 *src = reinterpret_cast<const float2 *>(out_s) + q;
 #pragma unroll
-            for (int i = 0; i < PPT; ++i) {
-                const int q = threadIdx.x + i * TT;
-                const int tj = q / PPT, v2 = 2 * (q - tj * PPT);
-                const int lim = tile_lim[tj];
-                if (u < (lim >> 4) && v2 < (lim & 15)) {    // W even: both columns or none
-                    const size_t off = (size_t)tile_base[tj] + (size_t)u * g.W + v2;
-                    if (EPI && out_half) *reinterpret_cast<uint32_t *>(yh + off) = to_bits16x2(row[q].x, row[q].y, out_half);
-                    else *reinterpret_cast<float2 *>(y + off) = row[q];
+            for (int u = 0; u < M; ++u) {
+                if (u < rows) {
+                    const float2 r = src[u * TT * PPT];
+                    if (EPI && out_half) *reinterpret_cast<uint32_t *>(yh + off) = to_bits16x2(r.x, r.y, out_half);
+                    else *reinterpret_cast<float2 *>(y + off) = r;
                 }
+                off += g.W;
             }
         }
     } else {
