@@ -171,6 +171,7 @@ wfq_status_t wfq_plan_create(wfq_plan_t **out, int N, int C, int K, int H, int W
     g.N = N; g.C = C; g.K = K; g.H = H; g.W = W;
     g.m = m; g.n = m + 2; g.P = g.n * g.n;
     g.TH = (H + m - 1) / m; g.TW = (W + m - 1) / m;
+    g.by_TH = wfq::FastDiv(g.TH); g.by_TW = wfq::FastDiv(g.TW);
     const long long T = (long long)N * g.TH * g.TW;
     const long long lim = (1LL << 31) - 1;
     if (T > lim || (long long)g.P * T * C > lim || (long long)g.P * K * C > lim ||

@@ -122,9 +122,9 @@ input_transform_int_kernel(const Tin *__restrict__ x, int8_t *__restrict__ Xq, f
     const int ng = prm.CB / gs, gs32 = gs >> 5;
 
     auto stage_item = [&](int item, int buf) {
-        const int cblk = item % prm.NCB, rest = item / prm.NCB;
-        const int srow = rest / prm.NCH, chunk = rest - srow * prm.NCH;
-        const int img = srow / g.TH, th = srow - img * g.TH;
+        const int rest = item / prm.by_NCB, cblk = item - rest * prm.NCB;
+        const int srow = rest / prm.by_NCH, chunk = rest - srow * prm.NCH;
+        const int img = srow / g.by_TH, th = srow - img * g.TH;
         const int first = chunk * prm.TB * M - 1;
         const int w_base = prm.vec16 ? ((first + 8) & ~7) - 8 : first - 1;
         stage_strip<Tin, NN>(reinterpret_cast<Tin *>(smem_raw + buf * prm.strip_bytes), x, g, prm, img,
@@ -149,8 +149,8 @@ input_transform_int_kernel(const Tin *__restrict__ x, int8_t *__restrict__ Xq, f
         __syncthreads();
 
         const Tin *strip = reinterpret_cast<const Tin *>(smem_raw + buf * prm.strip_bytes);
-        const int cblk = item % prm.NCB, rest = item / prm.NCB;
-        const int srow = rest / prm.NCH, chunk = rest - srow * prm.NCH;   // srow = img*TH + th
+        const int rest = item / prm.by_NCB, cblk = item - rest * prm.NCB;
+        const int srow = rest / prm.by_NCH, chunk = rest - srow * prm.NCH;   // srow = img*TH + th
         const int tw0 = chunk * prm.TB;
         const int ntile = min(prm.TB, g.TW - tw0);
         const int c_base = cblk * prm.CB;
@@ -161,7 +161,7 @@ input_transform_int_kernel(const Tin *__restrict__ x, int8_t *__restrict__ Xq, f
         };
 
         for (int wt = warp; wt < ntile * cb32; wt += NWARP) {
-            const int tl = wt / cb32, c32 = wt - tl * cb32;
+            const int tl = wt / prm.by_cb32, c32 = wt - tl * cb32;
             float d[NN][NN], m = 0.f;
             patch(tl, c32 * 32 + lane, d);
 #pragma unroll
@@ -173,7 +173,7 @@ input_transform_int_kernel(const Tin *__restrict__ x, int8_t *__restrict__ Xq, f
         }
         __syncthreads();
         for (int wt = warp; wt < ntile * cb32; wt += NWARP) {
-            const int tl = wt / cb32, c32 = wt - tl * cb32;
+            const int tl = wt / prm.by_cb32, c32 = wt - tl * cb32;
             const int c = c32 * 32 + lane;
             float amax = 0.f;                                    // of the group of these 32 channels
             for (int k = c32 / gs32 * gs32, e = k + gs32; k < e; ++k) amax = fmaxf(amax, amax_s[tl][k]);
@@ -209,7 +209,7 @@ input_transform_int_kernel(const Tin *__restrict__ x, int8_t *__restrict__ Xq, f
         __syncthreads();
         if (!prm.dbuf && next < prm.items) stage_item(next, 0);   // the strip buffer is free: refill it now
 
-        quantize_item<P, GSR, SPLIT, false>(Zs, CBP, ntile, ng, gs, srow, tw0, c_base, g, ScaleTables{}, Xq, sX);
+        quantize_item<P, GSR, SPLIT, false>(Zs, CBP, ntile, ng, gs, srow, tw0, c_base, g, InputScales{}, Xq, sX);
         __syncthreads();   // Z and this strip buffer are free again
     }
 }
@@ -312,7 +312,8 @@ output_transform_int_kernel(const float *__restrict__ Y, float *__restrict__ y, 
         }
     }
 
-    const int tw = t % g.TW, th = (t / g.TW) % g.TH, img = t / (g.TW * g.TH);
+    const int tq = t / g.by_TW, img = tq / g.by_TH;
+    const int tw = t - tq * g.TW, th = tq - img * g.TH;
     const int h0 = th * M, w0 = tw * M;
     const size_t base = (((size_t)img * g.K + k) * g.H + h0) * g.W + w0;
     auto row_of = [&](int u, float (&o)[M]) {

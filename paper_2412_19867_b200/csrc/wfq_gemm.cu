@@ -84,6 +84,7 @@ struct GemmArgs {
     int cg;                   // groups per chunk
     int items;                // work items: whole units, then the parts of the units that are cut (plan_gemm_units)
     int whole, parts;         // whole units, parts of a cut one
+    FastDiv by_NT, by_MT;     // blocks of columns and of rows
     float *Y;                 // [P][K][Tp]
     int32_t *acc_dump;        // [P][T][K][G] or null
     int *status;
@@ -101,14 +102,16 @@ __device__ __forceinline__ Item item_of(const GemmArgs &a, int i, int MT, int NT
     it.p0 = 0;
     it.np = BN / 16;
     if (CUT && i >= a.whole) {
-        const int r = i - a.whole;
-        i = a.whole + r / a.parts;
-        it.p0 = r % a.parts * part_pieces(BN);
+        constexpr int PARTS = BN / (16 * part_pieces(BN));
+        const int part = i - a.whole;
+        i = a.whole + part / PARTS;
+        it.p0 = part % PARTS * part_pieces(BN);
         it.np = part_pieces(BN);
     }
-    it.nt = i % NT;
-    it.mt = (i / NT) % MT;
-    it.p = i / (NT * MT);
+    const int r = i / a.by_NT;
+    it.nt = i - r * NT;
+    it.p = r / a.by_MT;
+    it.mt = r - it.p * MT;
     return it;
 }
 
@@ -554,7 +557,8 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         // The parts of cut units (at most one per CTA) run code of their own: a bound on the pieces inside the unrolled
         // loops keeps the compiler from interleaving them (all layers 10 % slower)
         for (int i = blockIdx.x; i < a.whole && ok; i += gridDim.x) {
-            const int nt = i % NT, mt = (i / NT) % MT, p = i / (NT * MT);
+            const int r = i / a.by_NT, p = r / a.by_MT;
+            const int nt = i - r * NT, mt = r - p * MT;
             ok = epilogue_unit<BN, SWAP, DUMP, CUT, BN / 16>(sh, tmY, a, g, ctx, ec, p, mt, nt * BN, 0, slot, sphase);
         }
         const int tail = a.whole + (int)blockIdx.x;
@@ -609,6 +613,8 @@ cudaError_t launch_variant(const wfq_plan &plan, int32_t *acc_dump, cudaStream_t
     a.whole = DUMP ? units : plan.gemm_whole;     // the debug output is not cut
     a.parts = DUMP ? 1 : plan.gemm_parts;
     a.items = a.whole + (units - a.whole) * a.parts;
+    a.by_NT = plan.gemm_by_nt;
+    a.by_MT = plan.gemm_by_mt;
     const int grid = a.items < slots ? a.items : slots;
     // the filters share L2 (126 MB) with Xq, sX and Y: at most 48 MB of them are asked for early
     a.l2_prefetch_bytes = pdl ? (48LL << 20) / grid : 0;
@@ -757,6 +763,8 @@ bool plan_gemm_units(wfq_plan &plan)
     const bool cut = parts > 1 && rest > 0 && parts * rest <= slots && (g.G + cg - 1) / cg > 1 && cols > part;
     plan.gemm_whole = cut ? units - rest : units;
     plan.gemm_parts = cut ? parts : 1;
+    plan.gemm_by_nt = FastDiv((cols + bn - 1) / bn);
+    plan.gemm_by_mt = FastDiv((rows + BM - 1) / BM);
     const unsigned long long dims[3] = {(unsigned long long)g.T, (unsigned long long)g.K, (unsigned long long)g.P};
     const unsigned long long strides[2] = {(unsigned long long)g.Tp * 4, (unsigned long long)g.K * g.Tp * 4};
     const unsigned box[3] = {32u, (unsigned)(cut ? part : bn), 1u};

@@ -160,7 +160,7 @@ __device__ __forceinline__ void transform_patch(float (&d)[NN][NN], float *__res
 template <int M, typename Tin, int GSR, int SPLIT>
 __global__ void __launch_bounds__(K1_THREADS, 4)
 input_transform_kernel(const Tin *__restrict__ x, int8_t *__restrict__ Xq,
-                       float *__restrict__ sX, Geometry g, ScaleTables tab, K1Params prm)
+                       float *__restrict__ sX, Geometry g, InputScales tab, K1Params prm)
 {
     constexpr int NN = M + 2;
     constexpr int P = NN * NN;
@@ -189,9 +189,9 @@ input_transform_kernel(const Tin *__restrict__ x, int8_t *__restrict__ Xq,
     // item -> (tile row, chunk of tiles, channel block); channel blocks vary fastest so
     // that CTAs running side by side read the same image rows
     auto stage_item = [&](int item, int buf) {
-        const int cblk = item % prm.NCB, rest = item / prm.NCB;
-        const int srow = rest / prm.NCH, chunk = rest - srow * prm.NCH;
-        const int img = srow / g.TH, th = srow - img * g.TH;
+        const int rest = item / prm.by_NCB, cblk = item - rest * prm.NCB;
+        const int srow = rest / prm.by_NCH, chunk = rest - srow * prm.NCH;
+        const int img = srow / g.by_TH, th = srow - img * g.TH;
         // first staged column: two left of the first tile's first output column, or (16-byte
         // pieces) the multiple of 8 at or below the first input column
         const int first = chunk * prm.TB * M - 1;
@@ -220,8 +220,8 @@ input_transform_kernel(const Tin *__restrict__ x, int8_t *__restrict__ Xq,
         __syncthreads();
 
         const Tin *strip = reinterpret_cast<const Tin *>(smem_raw + buf * prm.strip_bytes);
-        const int cblk = item % prm.NCB, rest = item / prm.NCB;
-        const int srow = rest / prm.NCH, chunk = rest - srow * prm.NCH;   // srow = img*TH + th
+        const int rest = item / prm.by_NCB, cblk = item - rest * prm.NCB;
+        const int srow = rest / prm.by_NCH, chunk = rest - srow * prm.NCH;   // srow = img*TH + th
         const int tw0 = chunk * prm.TB;
         const int ntile = min(prm.TB, g.TW - tw0);
         const int c_base = cblk * prm.CB;
@@ -229,7 +229,7 @@ input_transform_kernel(const Tin *__restrict__ x, int8_t *__restrict__ Xq,
         // ---- phase 1: transform, one (tile, channel) per thread ----------------------
         const int voff = tw0 * M - 2 - (((tw0 * M - 1 + 8) & ~7) - 8);   // 16-byte pieces: column of tile 0 minus one
         for (int wt = warp; wt < ntile * cb32; wt += NWARP) {
-            const int tl = wt / cb32;
+            const int tl = wt / prm.by_cb32;
             const int c = (wt - tl * cb32) * 32 + lane;
             float d[NN][NN];
             if (sizeof(Tin) == 2 && prm.vec16) load_patch_vec<NN>(strip + c * prm.CS, tl * M + voff, d);
@@ -259,7 +259,7 @@ struct K1NhwcShared {
 template <int M, typename Tin, int GSR, int SPLIT>
 __global__ void __launch_bounds__(K1_THREADS, 4)
 input_transform_nhwc_kernel(const __grid_constant__ CUtensorMap tmx, int8_t *__restrict__ Xq,
-                            float *__restrict__ sX, Geometry g, ScaleTables tab, K1Params prm, int *status,
+                            float *__restrict__ sX, Geometry g, InputScales tab, K1Params prm, int *status,
                             long long wait_cycles)
 {
     constexpr int NN = M + 2;
@@ -293,9 +293,9 @@ input_transform_nhwc_kernel(const __grid_constant__ CUtensorMap tmx, int8_t *__r
 
     // thread 0 only
     auto issue = [&](int item, int buf) {
-        const int cblk = item % prm.NCB, rest = item / prm.NCB;
-        const int srow = rest / prm.NCH, chunk = rest - srow * prm.NCH;
-        const int img = srow / g.TH, th = srow - img * g.TH;
+        const int rest = item / prm.by_NCB, cblk = item - rest * prm.NCB;
+        const int srow = rest / prm.by_NCH, chunk = rest - srow * prm.NCH;
+        const int img = srow / g.by_TH, th = srow - img * g.TH;
         const uint32_t bar = ptx::smem_u32(&sh.full[buf]);
         ptx::mbar_arrive_expect_tx(bar, box_bytes);
         ptx::tma_load_4d(ptx::smem_u32(smem_raw + buf * prm.strip_bytes), &tmx, bar, cblk * prm.CB,
@@ -318,15 +318,15 @@ input_transform_nhwc_kernel(const __grid_constant__ CUtensorMap tmx, int8_t *__r
         if (!ok) break;
 
         const Tin *strip = reinterpret_cast<const Tin *>(smem_raw + buf * prm.strip_bytes);
-        const int cblk = item % prm.NCB, rest = item / prm.NCB;
-        const int srow = rest / prm.NCH, chunk = rest - srow * prm.NCH;
+        const int rest = item / prm.by_NCB, cblk = item - rest * prm.NCB;
+        const int srow = rest / prm.by_NCH, chunk = rest - srow * prm.NCH;
         const int tw0 = chunk * prm.TB;
         const int ntile = min(prm.TB, g.TW - tw0);
         const int c_base = cblk * prm.CB;
 
         // ---- phase 1: transform, one (tile, channel) per thread ----------------------
         for (int wt = warp; wt < ntile * cb32; wt += NWARP) {
-            const int tl = wt / cb32;
+            const int tl = wt / prm.by_cb32;
             const int c = (wt - tl * cb32) * 32 + lane;
             float d[NN][NN];
             const Tin *src = strip + (size_t)(tl * M) * prm.CB + c;
@@ -500,6 +500,9 @@ void plan_k1(wfq_plan &plan, K1Params &prm, bool vec16, ResidentFn resident_of)
     prm.smem = (int)smem_bytes();
     prm.NCB = g.C / prm.CB;
     prm.items = g.N * g.TH * prm.NCH * prm.NCB;
+    prm.by_NCH = FastDiv(prm.NCH);
+    prm.by_NCB = FastDiv(prm.NCB);
+    prm.by_cb32 = FastDiv(prm.CB / 32);
     // persistent CTAs: as many as fit on the device at once
     const int per_sm = resident_of(plan, (size_t)prm.smem);
     const int resident = per_sm * (plan.sm_count > 0 ? plan.sm_count : 1);
@@ -538,6 +541,9 @@ static void plan_k1_nhwc(wfq_plan &plan)
     prm.smem = (int)smem_bytes();
     prm.NCB = g.C / prm.CB;
     prm.items = g.N * g.TH * prm.NCH * prm.NCB;
+    prm.by_NCH = FastDiv(prm.NCH);
+    prm.by_NCB = FastDiv(prm.NCB);
+    prm.by_cb32 = FastDiv(prm.CB / 32);
     const int per_sm = (int)k1_op(kK1nResident, M, f16, g.gs, nullptr, nullptr, nullptr, (size_t)prm.smem);
     const int resident = per_sm * (plan.sm_count > 0 ? plan.sm_count : 1);
     prm.grid = prm.items < resident ? prm.items : resident;

@@ -184,7 +184,7 @@ __device__ __noinline__ bool wait_counter(volatile int *ctr, uint32_t tick, int 
 
 template <int M, int GS, int MODE>
 __global__ void __launch_bounds__(TC_THREADS, 1)
-input_transform_tc_kernel(const __grid_constant__ CUtensorMap tmx, TcArgs a, Geometry g, ScaleTables tab)
+input_transform_tc_kernel(const __grid_constant__ CUtensorMap tmx, TcArgs a, Geometry g, InputScales tab)
 {
     using C = TcCfg<M>;
     constexpr int NN = C::NN, P = C::P, S = C::S, PL = C::PL, KSTEPS = C::KSTEPS;

@@ -101,12 +101,13 @@ struct TnArgs {
     long long wait_cycles;
     const uint4 *amat;        // the constant matrix as it lies in shared memory, AMAT_BYTES
     int NCH, NCB, items;      // chunks of TB tiles per tile row, channel blocks, work items
+    FastDiv by_NCH, by_NCB;
     int debug_skip_item;      // >= 0: the producer skips this item's copies (exercises the bounded waits)
 };
 
 template <int M, int GS>
 __global__ void __launch_bounds__((TnCfg<M, GS>::THREADS), 2)
-input_transform_tcn_kernel(const __grid_constant__ CUtensorMap tmx, TnArgs a, Geometry g, ScaleTables tab)
+input_transform_tcn_kernel(const __grid_constant__ CUtensorMap tmx, TnArgs a, Geometry g, InputScales tab)
 {
     using C = TnCfg<M, GS>;
     constexpr int TN_NSTRIP = C::NSTRIP, TN_NACC = C::NACC, TN_TEAMS = C::TEAMS, TN_THREADS = C::THREADS;
@@ -170,9 +171,9 @@ input_transform_tcn_kernel(const __grid_constant__ CUtensorMap tmx, TnArgs a, Ge
                                                       kWaitStripEmpty));
             if (!ok) break;
             if (lane == 0 && item != a.debug_skip_item) {
-                const int cblk = item % a.NCB, rest = item / a.NCB;
-                const int srow = rest / a.NCH, chunk = rest - srow * a.NCH;
-                const int img = srow / g.TH, th = srow - img * g.TH;
+                const int rest = item / a.by_NCB, cblk = item - rest * a.NCB;
+                const int srow = rest / a.by_NCH, chunk = rest - srow * a.NCH;
+                const int img = srow / g.by_TH, th = srow - img * g.TH;
                 const uint32_t bar = ptx::smem_u32(&sh.strip_full[sb]);
                 ptx::mbar_arrive_expect_tx(bar, (uint32_t)C::STRIP_BYTES);
 #pragma unroll
@@ -252,8 +253,8 @@ input_transform_tcn_kernel(const __grid_constant__ CUtensorMap tmx, TnArgs a, Ge
             const uint32_t aphase = (uint32_t)(j / TN_NACC) & 1u;
             if (!wait_bounded(ptx::smem_u32(&sh.acc_full[slot]), aphase, ctx, kWaitAccFull)) break;
             ptx::tc_fence_after();
-            const int cblk = item % a.NCB, rest = item / a.NCB;
-            const int srow = rest / a.NCH, chunk = rest - srow * a.NCH;
+            const int rest = item / a.by_NCB, cblk = item - rest * a.NCB;
+            const int srow = rest / a.by_NCH, chunk = rest - srow * a.NCH;
             const int tw = chunk * C::TB + tl;
             const bool valid = row_ok && tw < g.TW;
             const int t = srow * g.TW + tw;
@@ -382,6 +383,8 @@ cudaError_t launch_tn(const wfq_plan &plan, cudaStream_t stream)
     a.amat = static_cast<const uint4 *>(g_tn_amat[plan.device][M == 6 ? 1 : 0]);
     a.NCH = (g.TW + C::TB - 1) / C::TB;
     a.NCB = g.C / C::ACC_COLS;
+    a.by_NCH = FastDiv(a.NCH);
+    a.by_NCB = FastDiv(a.NCB);
     a.items = g.N * g.TH * a.NCH * a.NCB;
     a.debug_skip_item = plan.debug_skip_item;
     if (!a.amat) return cudaErrorInvalidValue;

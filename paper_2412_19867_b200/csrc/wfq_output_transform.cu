@@ -59,7 +59,7 @@ constexpr int kEarlyFlag = 4;
 template <int M, int STORE, bool EPI, int TT, int LOAD>
 __global__ void __launch_bounds__(TT, (M == 6 ? (EPI ? 6 : 7) : 8) * 128 / TT)
 output_transform_kernel(const float *__restrict__ Y, float *__restrict__ y, Geometry g,
-                        ScaleTables tab, const float *__restrict__ bias, int act, int flags)
+                        OutputScales tab, const float *__restrict__ bias, int act, int flags)
 {
     constexpr int NN = M + 2;
     const int out_half = flags & (kEarlyFlag - 1);
@@ -104,12 +104,9 @@ output_transform_kernel(const float *__restrict__ Y, float *__restrict__ y, Geom
 #pragma unroll
             for (int u = 0; u < M; ++u) tmp[u][j] = o[u];
         }
-        const int tw = t % g.TW;
-        const int tq = t / g.TW;
-        const int th = tq % g.TH;
-        const int img = tq / g.TH;
-        h0 = th * M;
-        w0 = tw * M;
+        const int tq = t / g.by_TW, img = tq / g.by_TH;
+        h0 = (tq - img * g.TH) * M;
+        w0 = (t - tq * g.TW) * M;
         base = (((size_t)img * g.K + k) * g.H + h0) * g.W + w0;
     }
 

@@ -252,7 +252,7 @@ __device__ __forceinline__ void group_scale(float amax, float &scale, float &inv
 template <int P, int GSR, int SPLIT, bool SCALED = true>
 __device__ __forceinline__ void quantize_item(const float *__restrict__ Zs, int CBP, int ntile, int ng, int gs,
                                               int srow, int tw0, int c_base, const Geometry &g,
-                                              const ScaleTables &tab, int8_t *__restrict__ Xq,
+                                              const InputScales &tab, int8_t *__restrict__ Xq,
                                               float *__restrict__ sX)
 {
     // X = Z * (caller's per-position factor) is formed here, one rounding, as the
@@ -267,7 +267,7 @@ __device__ __forceinline__ void quantize_item(const float *__restrict__ Zs, int 
             const int tk = act ? task : 0;
             const int part = tk % SPLIT, rest = tk / SPLIT;
             const int q = rest / P, p = rest - q * P;
-            const int tl = q / ng, grp = q - tl * ng;
+            const int tl = q >> (ng - 1), grp = q - tl * ng;        // one or two groups per item
             const int t = srow * g.TW + tw0 + tl;
             const float4 *src = reinterpret_cast<const float4 *>(Zs + (size_t)(tl * P + p) * CBP + grp * gs +
                                                                  part * GSR);
@@ -299,7 +299,7 @@ __device__ __forceinline__ void quantize_item(const float *__restrict__ Zs, int 
         const int tasks = ntile * ng * P;
         for (int task = threadIdx.x; task < tasks; task += K1_THREADS) {
             const int q = task / P, p = task - q * P;
-            const int tl = q / ng, grp = q - tl * ng;
+            const int tl = q >> (ng - 1), grp = q - tl * ng;        // one or two groups per item
             const int t = srow * g.TW + tw0 + tl;
             const float4 *src = reinterpret_cast<const float4 *>(Zs + (size_t)(tl * P + p) * CBP + grp * gs);
             int8_t *dst = Xq + ((size_t)p * g.T + t) * g.C + c_base + grp * gs;
