@@ -133,12 +133,11 @@ input_transform_int_kernel(const Tin *__restrict__ x, int8_t *__restrict__ Xq, f
     };
 
     int item = blockIdx.x;
-    if (prm.dbuf && item < prm.items) stage_item(item, 0);
+    if (item < prm.items) stage_item(item, 0);
     for (int it = 0; item < prm.items; ++it, item += gridDim.x) {
         const int buf = prm.dbuf ? (it & 1) : 0;
         const int next = item + gridDim.x;
         if (!prm.dbuf) {
-            if (it == 0) stage_item(item, 0);
             cp_async_wait_group<0>();
         } else if (next < prm.items) {
             stage_item(next, buf ^ 1);
