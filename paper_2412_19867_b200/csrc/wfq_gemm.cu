@@ -555,7 +555,7 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         const EpiCtx ec{tmem_base + ((uint32_t)(quarter * 32) << 16), scales,
                         store + quarter * (C::STORE_BYTES / NUM_EPI_WARPS), quarter, lane, nchunk};
         // The parts of cut units (at most one per CTA) run code of their own: a bound on the pieces inside the unrolled
-        // loops keeps the compiler from interleaving them (all layers 10 % slower)
+        // loops keeps the compiler from interleaving them (34 layers 5 % slower, up to 13 %)
         for (int i = blockIdx.x; i < a.whole && ok; i += gridDim.x) {
             const int r = i / a.by_NT, p = r / a.by_MT;
             const int nt = i - r * NT, mt = r - p * MT;

@@ -56,8 +56,12 @@ __device__ __forceinline__ void at_1d(const float (&v)[M + 2], float (&o)[M])
 // flags: output type (0 fp32, 1 fp16, 2 bf16), plus kEarlyFlag.  One argument for both: a further one makes a launch
 // longer (layers of 12.2 us that wait for launches 12.7 us).
 constexpr int kEarlyFlag = 4;
+// F(6,3): registers for five CTAs of 128 tiles per SM (89 to 96) instead of seven (72; six with an epilogue, 80).  The
+// 64 loads of a thread then stand further ahead of the arithmetic, and most layers are one wave of fewer CTAs anyway
+// (forward, 36 tiles x 1280 channels 41.5 -> 40.6 us, 925 x 48 16.8 -> 16.0 us, 126 x 256 16.5 -> 16.2 us; several waves,
+// 3200 x 64, 40.1 -> 40.2 us).  Four CTAs (125 registers) are no better, nor are six for F(4,3).
 template <int M, int STORE, bool EPI, int TT, int LOAD>
-__global__ void __launch_bounds__(TT, (M == 6 ? (EPI ? 6 : 7) : 8) * 128 / TT)
+__global__ void __launch_bounds__(TT, (M == 6 ? 5 : 8) * 128 / TT)
 output_transform_kernel(const float *__restrict__ Y, float *__restrict__ y, Geometry g,
                         OutputScales tab, const float *__restrict__ bias, int act, int flags)
 {
@@ -134,8 +138,8 @@ bool evict_early(const wfq_plan &plan)
 }
 // With two forms of the loads in the kernel the compiler issues all of them before the arithmetic, which is faster
 // than one form scheduled into it (forward, 600 tiles of 320 channels 35.5 -> 34.5 us, 243 of 128 14.2 -> 13.8 us, F(4,3)
-// 2048 of 128 24.3 -> 24.0 us).  The F(6,3) variants with an epilogue have no registers for it (80 with 4 to 16 bytes
-// spilled; 256 tiles of 1280 channels 80.9 us, with one form 75.8 us).
+// 2048 of 128 24.3 -> 24.0 us).  The F(6,3) variants with an epilogue are better off with one form (1600 tiles of 128
+// channels 34.4 us, with two 35.4 us).
 constexpr bool both_loads(int m, bool epi, int tt) { return tt == 128 && !(m == 6 && epi); }
 
 template <int M, int STORE, bool EPI, int TT>
