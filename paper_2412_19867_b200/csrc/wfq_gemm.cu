@@ -24,12 +24,13 @@
 //            scales, then per group tcgen05.ld the int32 sums, convert and scale into fp32
 //            registers (packed f32x2 multiply / fma), release the slot; after the last
 //            chunk of a unit write Y[p][k][t].
-// The second CTA of the SM runs the same pipeline on other units, which hides the
-// hand-over latencies and overlaps one CTA's output stores with the other's arithmetic.
-// Only four epilogue warps per CTA on purpose: the warp schedulers share issue slots
-// evenly among ready warps, so every additional arithmetic warp slows the three
-// single-purpose warps whose few instructions sit on the critical path (measured:
-// 8 epilogue warps per CTA were 15-25 % slower).
+// The second CTA of the SM runs the same pipeline on other units, which hides part of the
+// hand-over latencies; the stores of Y leave through the TMA unit (rows = tiles).
+// What bounds it: a chunk of 2 x 64 columns takes an epilogue warp 541 cycles alone and 867 beside
+// the other CTA's (784 for both at the full rate of its arithmetic), and some 300 more pass between
+// chunks; 14x14 with groups of 32, 1024 tiles x 256 channels: 16 us for 75 M group sums and 50 MB.
+// Four epilogue warps per CTA: eight, with half of the columns each, are 1 % slower (forward, ten
+// layers), and the registers for 64 sums and two blocks of 16 leave no room for more.
 // Every wait is bounded; on expiry the CTA records where, stops, drains and frees TMEM.
 #include "wfq_internal.h"
 #include "wfq_ptx.cuh"
