@@ -214,7 +214,9 @@ __device__ __forceinline__ bool epilogue_unit(Shared *sh, const CUtensorMap &tmY
 
     for (int ch = 0; ch < ec.nchunk; ++ch) {
         const int g0 = ch * a.cg, ng = min(a.cg, g.G - g0);
-        if (!wait_bounded(ptx::smem_u32(&sh->acc_full[slot]), sphase, ctx, kWaitTmemFull)) return false;
+        // the warp gives up as a whole: tcgen05.ld and elect.sync below need all of its lanes
+        if (!__all_sync(0xffffffffu, wait_bounded(ptx::smem_u32(&sh->acc_full[slot]), sphase, ctx, kWaitTmemFull)))
+            return false;
         if (active) {
             ptx::tc_fence_after();
             const float *sc = ec.scales + (size_t)slot * C::SLOT_SCALE_FLOATS;

@@ -490,7 +490,9 @@ input_transform_tc_kernel(const __grid_constant__ CUtensorMap tmx, TcArgs a, Geo
         }
         for (int grp = team; grp < ngroups; grp += TC_TEAMS) {
             const int acc = team;                          // TC_NACC == TC_TEAMS
-            if (!wait_bounded(ptx::smem_u32(&sh->acc_full[acc]), (uint32_t)((grp / TC_NACC) & 1), ctx, kWaitAccFull))
+            // the warp gives up as a whole: tcgen05.ld below needs all of its lanes
+            if (!__all_sync(0xffffffffu, wait_bounded(ptx::smem_u32(&sh->acc_full[acc]),
+                                                      (uint32_t)((grp / TC_NACC) & 1), ctx, kWaitAccFull)))
                 break;
             ptx::tc_fence_after();
             const uint32_t taddr = taddr0 + (uint32_t)(acc * 128);

@@ -251,7 +251,9 @@ input_transform_tcn_kernel(const __grid_constant__ CUtensorMap tmx, TnArgs a, Ge
         for (int item = blockIdx.x + team * stride; item < a.items; item += TN_TEAMS * stride, j += TN_TEAMS) {
             const int slot = j % TN_NACC;
             const uint32_t aphase = (uint32_t)(j / TN_NACC) & 1u;
-            if (!wait_bounded(ptx::smem_u32(&sh.acc_full[slot]), aphase, ctx, kWaitAccFull)) break;
+            // the warp gives up as a whole: tcgen05.ld below needs all of its lanes
+            if (!__all_sync(0xffffffffu, wait_bounded(ptx::smem_u32(&sh.acc_full[slot]), aphase, ctx, kWaitAccFull)))
+                break;
             ptx::tc_fence_after();
             const int rest = item / a.by_NCB, cblk = item - rest * a.NCB;
             const int srow = rest / a.by_NCH, chunk = rest - srow * a.NCH;
