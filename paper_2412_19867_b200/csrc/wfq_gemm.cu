@@ -141,15 +141,14 @@ __device__ __forceinline__ void mma_issue_aligned(Shared *sh, uint32_t tiles_lo,
         const uint32_t idesc = ptx::idesc_i8(BM, 16 * it.np);
         for (int kb = 0; kb < KB; ++kb) {
             const int nslice = kb == KB - 1 ? last_slices : BK / UK;
-            if (!__all_sync(0xffffffffu, wait_bounded(full0 + 8u * stage, phase, ctx, kWaitSmemFull)))
+            if (!wait_warp(full0 + 8u * stage, phase, ctx, kWaitSmemFull))
                 return;
             const uint32_t a_lo = tiles_lo + (uint32_t)(stage * (C::STAGE_BYTES >> 4));
             const uint32_t b_lo = a_lo + (uint32_t)(A_BYTES >> 4) + (uint32_t)(it.p0 * (16 * BK >> 4));
 #pragma unroll
             for (int c = 0; c < NCH; ++c) {
                 if (c * CHUNK_STEPS < nslice) {           // the chunk has at least one group
-                    if (!__all_sync(0xffffffffu, wait_bounded(free0 + 8u * slot, sphase ^ 1u, ctx,
-                                                              kWaitTmemEmpty)))
+                    if (!wait_warp(free0 + 8u * slot, sphase ^ 1u, ctx, kWaitTmemEmpty))
                         return;
                     ptx::tc_fence_after();
                     if (ptx::elect_one()) {
@@ -214,9 +213,7 @@ __device__ __forceinline__ bool epilogue_unit(Shared *sh, const CUtensorMap &tmY
 
     for (int ch = 0; ch < ec.nchunk; ++ch) {
         const int g0 = ch * a.cg, ng = min(a.cg, g.G - g0);
-        // the warp gives up as a whole: tcgen05.ld and elect.sync below need all of its lanes
-        if (!__all_sync(0xffffffffu, wait_bounded(ptx::smem_u32(&sh->acc_full[slot]), sphase, ctx, kWaitTmemFull)))
-            return false;
+        if (!wait_warp(ptx::smem_u32(&sh->acc_full[slot]), sphase, ctx, kWaitTmemFull)) return false;
         if (active) {
             ptx::tc_fence_after();
             const float *sc = ec.scales + (size_t)slot * C::SLOT_SCALE_FLOATS;
@@ -402,8 +399,7 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             const Item it = item_of<BN, CUT>(a, i, MT, NT);
             const int nt = it.nt, mt = it.mt, p = it.p;
             for (int kb = 0; kb < KB; ++kb) {
-                ok = __all_sync(0xffffffffu, wait_bounded(ptx::smem_u32(&sh->empty[stage]), phase ^ 1u, ctx,
-                                                          kWaitSmemEmpty));
+                ok = wait_warp(ptx::smem_u32(&sh->empty[stage]), phase ^ 1u, ctx, kWaitSmemEmpty);
                 if (!ok) break;
                 if (ptx::elect_one() && !(blockIdx.x == 0 && issued == a.debug_skip_stage)) {
                     const uint32_t bar = ptx::smem_u32(&sh->full[stage]);
@@ -464,8 +460,7 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             int in_group = 0;      // MMA step within the group
             uint32_t dcol = 0;     // TMEM column of the current group
             for (int kb = 0; kb < KB && ok; ++kb) {
-                ok = __all_sync(0xffffffffu, wait_bounded(ptx::smem_u32(&sh->full[stage]), phase, ctx,
-                                                          kWaitSmemFull));
+                ok = wait_warp(ptx::smem_u32(&sh->full[stage]), phase, ctx, kWaitSmemFull);
                 if (!ok) break;
                 ptx::tc_fence_after();
                 // a 32-byte step along K inside the swizzled rows is +2 in the address field
@@ -475,8 +470,7 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 for (int s = 0; s < nslice; ++s) {
                     if (step == 0) {
                         // start of a chunk: its TMEM slot must have been drained
-                        ok = __all_sync(0xffffffffu, wait_bounded(ptx::smem_u32(&sh->slot_free[slot]),
-                                                                  sphase ^ 1u, ctx, kWaitTmemEmpty));
+                        ok = wait_warp(ptx::smem_u32(&sh->slot_free[slot]), sphase ^ 1u, ctx, kWaitTmemEmpty);
                         if (!ok) break;
                         ptx::tc_fence_after();
                         dcol = tmem_base + (uint32_t)(slot * SLOT_COLS);
@@ -517,8 +511,7 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 const int nt = it.nt, mt = it.mt, p = it.p;
                 for (int ch = 0; ch < nchunk; ++ch) {
                     const int g0 = ch * cg, ng = min(cg, g.G - g0);
-                    ok = __all_sync(0xffffffffu, wait_bounded(ptx::smem_u32(&sh->slot_free[slot]), sphase ^ 1u,
-                                                              ctx, kWaitScaleEmpty));
+                    ok = wait_warp(ptx::smem_u32(&sh->slot_free[slot]), sphase ^ 1u, ctx, kWaitScaleEmpty);
                     if (!ok) break;
                     const uint32_t bar = ptx::smem_u32(&sh->acc_full[slot]);
                     const uint32_t dst = ptx::smem_u32(scales + (size_t)slot * C::SLOT_SCALE_FLOATS);
@@ -684,7 +677,7 @@ __global__ void __launch_bounds__(128, 1) mma_peak_kernel(int mmas, int *status,
             ptx::umma_commit(ptx::smem_u32(&sh->done));
         }
         __syncwarp();
-        wait_bounded(ptx::smem_u32(&sh->done), 0, ctx, kWaitTmemFull);
+        wait_warp(ptx::smem_u32(&sh->done), 0, ctx, kWaitTmemFull);
     }
     ptx::tc_fence_before();
     __syncthreads();

@@ -313,7 +313,7 @@ input_transform_nhwc_kernel(const __grid_constant__ CUtensorMap tmx, int8_t *__r
     for (; item < prm.items; ++it, item += stride) {
         const int buf = prm.dbuf ? (it & 1) : 0;
         const uint32_t parity = (uint32_t)(prm.dbuf ? (it >> 1) : it) & 1u;
-        ok = wait_bounded(ptx::smem_u32(&sh.full[buf]), parity, ctx, kWaitStripFull);
+        ok = wait_warp(ptx::smem_u32(&sh.full[buf]), parity, ctx, kWaitStripFull);
         if (!ok) break;
 
         const Tin *strip = reinterpret_cast<const Tin *>(smem_raw + buf * prm.strip_bytes);

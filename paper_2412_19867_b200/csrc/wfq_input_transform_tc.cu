@@ -265,8 +265,7 @@ input_transform_tc_kernel(const __grid_constant__ CUtensorMap tmx, TcArgs a, Geo
         bool ok = true;
         for (int item = blockIdx.x; item < a.items && ok; item += gridDim.x, ++k) {
             if (k >= prefilled) {
-                ok = __all_sync(0xffffffffu, wait_bounded(ptx::smem_u32(&sh->strip_empty[sidx]), phase ^ 1u, ctx,
-                                                          kWaitStripEmpty));
+                ok = wait_warp(ptx::smem_u32(&sh->strip_empty[sidx]), phase ^ 1u, ctx, kWaitStripEmpty);
                 if (!ok) break;
                 issue_strip(item, sidx);
                 __syncwarp();
@@ -288,13 +287,11 @@ input_transform_tc_kernel(const __grid_constant__ CUtensorMap tmx, TcArgs a, Geo
         const int npairs = (nbt + 1) >> 1;
         int slot = 0, s = 0, acc = 0;
         uint32_t phase = 0, aphase = 0;
-        bool have_a = __all_sync(0xffffffffu, wait_bounded(ptx::smem_u32(&sh->amat_full), 0, ctx, kWaitSmemFull));
+        bool have_a = wait_warp(ptx::smem_u32(&sh->amat_full), 0, ctx, kWaitSmemFull);
         for (int k = 0; k < npairs && have_a; ++k) {
-            if (!__all_sync(0xffffffffu, wait_bounded(ptx::smem_u32(&sh->pair_full[slot]), phase, ctx,
-                                                      kWaitPairFull)))
+            if (!wait_warp(ptx::smem_u32(&sh->pair_full[slot]), phase, ctx, kWaitPairFull))
                 break;
-            if (s == 0 && !__all_sync(0xffffffffu, wait_bounded(ptx::smem_u32(&sh->acc_empty[acc]),
-                                                                aphase ^ 1u, ctx, kWaitAccEmpty)))
+            if (s == 0 && !wait_warp(ptx::smem_u32(&sh->acc_empty[acc]), aphase ^ 1u, ctx, kWaitAccEmpty))
                 break;
             ptx::tc_fence_after();
             if (lane == 0) {
@@ -328,8 +325,7 @@ input_transform_tc_kernel(const __grid_constant__ CUtensorMap tmx, TcArgs a, Geo
         int slot = 0;
         uint32_t phase = 0;
         for (int k = 0; k < npairs; ++k) {
-            if (!__all_sync(0xffffffffu, wait_bounded(ptx::smem_u32(&sh->pair_empty[slot]), phase, ctx,
-                                                      kWaitPairEmpty)))
+            if (!wait_warp(ptx::smem_u32(&sh->pair_empty[slot]), phase, ctx, kWaitPairEmpty))
                 break;
             if (lane == 0) {
                 sh->pairs_consumed = k + 1;
@@ -353,8 +349,7 @@ input_transform_tc_kernel(const __grid_constant__ CUtensorMap tmx, TcArgs a, Geo
             // Every im2col warp waits for the strip, also one without a task in this item:
             // its arrival on strip_empty below must not run ahead of the producer, or it
             // would be counted for an earlier use of the same buffer.
-            ok = __all_sync(0xffffffffu, wait_bounded(ptx::smem_u32(&sh->strip_full[sidx]), sphase, ctx,
-                                                      kWaitStripFull));
+            ok = wait_warp(ptx::smem_u32(&sh->strip_full[sidx]), sphase, ctx, kWaitStripFull);
             for (int task = rw; task < ntask && ok; task += TC_READERS) {
                 const int tq = task / TC_CQ, cq = task - tq * TC_CQ;
                 const int bfirst = b0 + tq * 4;
@@ -490,9 +485,7 @@ input_transform_tc_kernel(const __grid_constant__ CUtensorMap tmx, TcArgs a, Geo
         }
         for (int grp = team; grp < ngroups; grp += TC_TEAMS) {
             const int acc = team;                          // TC_NACC == TC_TEAMS
-            // the warp gives up as a whole: tcgen05.ld below needs all of its lanes
-            if (!__all_sync(0xffffffffu, wait_bounded(ptx::smem_u32(&sh->acc_full[acc]),
-                                                      (uint32_t)((grp / TC_NACC) & 1), ctx, kWaitAccFull)))
+            if (!wait_warp(ptx::smem_u32(&sh->acc_full[acc]), (uint32_t)((grp / TC_NACC) & 1), ctx, kWaitAccFull))
                 break;
             ptx::tc_fence_after();
             const uint32_t taddr = taddr0 + (uint32_t)(acc * 128);

@@ -167,8 +167,7 @@ input_transform_tcn_kernel(const __grid_constant__ CUtensorMap tmx, TnArgs a, Ge
         long long issued = 0;
         bool ok = true;
         for (int item = blockIdx.x; item < a.items && ok; item += stride) {
-            ok = __all_sync(0xffffffffu, wait_bounded(ptx::smem_u32(&sh.strip_empty[sb]), phase ^ 1u, ctx,
-                                                      kWaitStripEmpty));
+            ok = wait_warp(ptx::smem_u32(&sh.strip_empty[sb]), phase ^ 1u, ctx, kWaitStripEmpty);
             if (!ok) break;
             if (lane == 0 && item != a.debug_skip_item) {
                 const int rest = item / a.by_NCB, cblk = item - rest * a.NCB;
@@ -206,10 +205,9 @@ input_transform_tcn_kernel(const __grid_constant__ CUtensorMap tmx, TnArgs a, Ge
         int sb = 0, slot = 0;
         uint32_t phase = 0, aphase = 0;
         for (int item = blockIdx.x; item < a.items; item += stride) {
-            if (!__all_sync(0xffffffffu, wait_bounded(ptx::smem_u32(&sh.strip_full[sb]), phase, ctx, kWaitStripFull)))
+            if (!wait_warp(ptx::smem_u32(&sh.strip_full[sb]), phase, ctx, kWaitStripFull))
                 break;
-            if (!__all_sync(0xffffffffu, wait_bounded(ptx::smem_u32(&sh.acc_empty[slot]), aphase ^ 1u, ctx,
-                                                      kWaitAccEmpty)))
+            if (!wait_warp(ptx::smem_u32(&sh.acc_empty[slot]), aphase ^ 1u, ctx, kWaitAccEmpty))
                 break;
             ptx::tc_fence_after();
             if (lane == 0) {
@@ -251,9 +249,7 @@ input_transform_tcn_kernel(const __grid_constant__ CUtensorMap tmx, TnArgs a, Ge
         for (int item = blockIdx.x + team * stride; item < a.items; item += TN_TEAMS * stride, j += TN_TEAMS) {
             const int slot = j % TN_NACC;
             const uint32_t aphase = (uint32_t)(j / TN_NACC) & 1u;
-            // the warp gives up as a whole: tcgen05.ld below needs all of its lanes
-            if (!__all_sync(0xffffffffu, wait_bounded(ptx::smem_u32(&sh.acc_full[slot]), aphase, ctx, kWaitAccFull)))
-                break;
+            if (!wait_warp(ptx::smem_u32(&sh.acc_full[slot]), aphase, ctx, kWaitAccFull)) break;
             ptx::tc_fence_after();
             const int rest = item / a.by_NCB, cblk = item - rest * a.NCB;
             const int srow = rest / a.by_NCH, chunk = rest - srow * a.NCH;

@@ -450,10 +450,13 @@ static __device__ __noinline__ bool wait_slow(uint32_t bar, uint32_t parity, con
         }
     }
 }
-__device__ __forceinline__ bool wait_bounded(uint32_t bar, uint32_t parity, const WaitCtx &ctx, int where)
+// The wait of a whole converged warp, with one answer for all of its lanes: a warp whose lanes gave up one by one would
+// leave some of them behind in an instruction that needs the others (tcgen05.ld, elect.sync) and has no limit.  The vote
+// on the first try makes the branch to the loop uniform.
+__device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, const WaitCtx &ctx, int where)
 {
-    if (ptx::mbar_try_wait(bar, parity)) return true;
-    return wait_slow(bar, parity, ctx, where);
+    if (__all_sync(0xffffffffu, ptx::mbar_try_wait(bar, parity))) return true;
+    return __all_sync(0xffffffffu, wait_slow(bar, parity, ctx, where));
 }
 // Bounded wait for copies that may still be in flight when a role gives up.
 __device__ __forceinline__ void drain(uint32_t bar, uint32_t parity, long long limit)
