@@ -59,6 +59,7 @@ struct Shared {
     uint64_t empty[NSTAGES];    // the MMAs reading a stage have completed
     uint64_t acc_full[NSLOT];      // the MMAs of a chunk have completed and its scales have landed
     uint64_t slot_free[NSLOT];     // all epilogue warps are done with a chunk
+    uint64_t mma_done;             // after a wait that ran out: every MMA issued has completed
     uint32_t tmem_base;
     volatile int abort;
 };
@@ -338,6 +339,7 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             ptx::mbar_init(ptx::smem_u32(&sh->acc_full[b]), DUMP ? 1 : 2);   // MMAs, scales
             ptx::mbar_init(ptx::smem_u32(&sh->slot_free[b]), NUM_EPI_WARPS);
         }
+        ptx::mbar_init(ptx::smem_u32(&sh->mma_done), 1);
         sh->abort = 0;
         ptx::fence_mbar_init();
     }
@@ -419,14 +421,14 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 if (++stage == NSTAGES) { stage = 0; phase ^= 1u; }
             }
         }
-        if (!ok) {
+        if (!ok || sh->abort) {
             // give copies still in flight a bounded time to land before the CTA exits
             int s = stage;
             uint32_t ph = phase;
             const long long n = issued < NSTAGES ? issued : NSTAGES;
             for (long long i = 0; i < n; ++i) {
                 if (--s < 0) { s = NSTAGES - 1; ph ^= 1u; }
-                drain(ptx::smem_u32(&sh->full[s]), ph, a.wait_cycles / 16);
+                drain(ptx::smem_u32(&sh->full[s]), ph);
             }
         }
     } else if (warp == 1) {
@@ -532,13 +534,13 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                     if (++slot == NSLOT) { slot = 0; sphase ^= 1u; }
                 }
             }
-            if (!ok) {
+            if (!ok || sh->abort) {      // where the chunk's MMAs were not issued this runs out its limit, the copies land
                 int s = slot;
                 uint32_t ph = sphase;
                 const long long n = issued < NSLOT ? issued : NSLOT;
                 for (long long i = 0; i < n; ++i) {
                     if (--s < 0) { s = NSLOT - 1; ph ^= 1u; }
-                    drain(ptx::smem_u32(&sh->acc_full[s]), ph, a.wait_cycles / 16);
+                    drain(ptx::smem_u32(&sh->acc_full[s]), ph);
                 }
             }
         }
@@ -572,6 +574,11 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     ptx::tc_fence_before();
     __syncthreads();
     if (warp == 1) {
+        if (sh->abort) {      // a wait ran out: MMAs may still be reading the stages and writing the accumulators
+            if (ptx::elect_one()) ptx::umma_commit(ptx::smem_u32(&sh->mma_done));
+            __syncwarp();
+            drain(ptx::smem_u32(&sh->mma_done), 0);
+        }
         ptx::tc_fence_after();
         ptx::tmem_dealloc(tmem_base, TMEM_COLS);
     }

@@ -349,7 +349,7 @@ input_transform_nhwc_kernel(const __grid_constant__ CUtensorMap tmx, int8_t *__r
         // shared memory goes away (copies issued: `issued`, consumed: `it`)
         for (int k = it; k < issued; ++k) {
             const int b = prm.dbuf ? (k & 1) : 0;
-            drain(ptx::smem_u32(&sh.full[b]), (uint32_t)(prm.dbuf ? (k >> 1) : k) & 1u, wait_cycles / 16);
+            drain(ptx::smem_u32(&sh.full[b]), (uint32_t)(prm.dbuf ? (k >> 1) : k) & 1u);
         }
     }
 }

@@ -272,12 +272,11 @@ input_transform_tc_kernel(const __grid_constant__ CUtensorMap tmx, TcArgs a, Geo
             }
             if (++sidx == a.nstrip) { sidx = 0; phase ^= 1u; }
         }
-        if (!ok) {
+        if (!ok || sh->abort) {
             // give copies still in flight a bounded time to land before the CTA exits
             const int issued = k > prefilled ? k : prefilled;
             for (int j = issued - 1; j >= 0 && j >= issued - a.nstrip; --j)
-                drain(ptx::smem_u32(&sh->strip_full[j % a.nstrip]), (uint32_t)((j / a.nstrip) & 1),
-                      a.wait_cycles / 16);
+                drain(ptx::smem_u32(&sh->strip_full[j % a.nstrip]), (uint32_t)((j / a.nstrip) & 1));
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
@@ -318,7 +317,7 @@ input_transform_tc_kernel(const __grid_constant__ CUtensorMap tmx, TcArgs a, Geo
         // unless a wait ran out)
         if (lane == 0) ptx::umma_commit(ptx::smem_u32(&sh->mma_done));
         __syncwarp();
-        drain(ptx::smem_u32(&sh->mma_done), 0, a.wait_cycles / 16);
+        drain(ptx::smem_u32(&sh->mma_done), 0);
     } else if (warp == 2) {
         // ---------------- retire: completed pairs, in order, as a counter ----------------
         const int npairs = (nbt + 1) >> 1;

@@ -90,6 +90,7 @@ struct TnShared {
     uint64_t strip_empty[TN_MAX_NSTRIP];
     uint64_t acc_full[TN_MAX_NACC];
     uint64_t acc_empty[TN_MAX_NACC];
+    uint64_t mma_done;       // after a wait that ran out: every MMA issued has completed
     uint32_t tmem_base;
     volatile int abort;
 };
@@ -128,6 +129,7 @@ input_transform_tcn_kernel(const __grid_constant__ CUtensorMap tmx, TnArgs a, Ge
             ptx::mbar_init(ptx::smem_u32(&sh.acc_full[s]), 1);
             ptx::mbar_init(ptx::smem_u32(&sh.acc_empty[s]), 4);
         }
+        ptx::mbar_init(ptx::smem_u32(&sh.mma_done), 1);
         sh.abort = 0;
         ptx::fence_mbar_init();
         ptx::prefetch_tmap(&tmx);
@@ -187,13 +189,13 @@ input_transform_tcn_kernel(const __grid_constant__ CUtensorMap tmx, TnArgs a, Ge
             ++issued;
             if (++sb == TN_NSTRIP) { sb = 0; phase ^= 1u; }
         }
-        if (!ok) {
+        if (!ok || sh.abort) {
             int s = sb;
             uint32_t ph = phase;
             const long long n = issued < TN_NSTRIP ? issued : TN_NSTRIP;
             for (long long i = 0; i < n; ++i) {
                 if (--s < 0) { s = TN_NSTRIP - 1; ph ^= 1u; }
-                drain(ptx::smem_u32(&sh.strip_full[s]), ph, a.wait_cycles / 16);
+                drain(ptx::smem_u32(&sh.strip_full[s]), ph);
             }
         }
     } else if (warp == 1) {
@@ -328,6 +330,11 @@ input_transform_tcn_kernel(const __grid_constant__ CUtensorMap tmx, TnArgs a, Ge
     ptx::tc_fence_before();
     __syncthreads();
     if (warp == 1) {
+        if (sh.abort) {       // a wait ran out: MMAs may still be reading the strips and writing the accumulators
+            if (lane == 0) ptx::umma_commit(ptx::smem_u32(&sh.mma_done));
+            __syncwarp();
+            drain(ptx::smem_u32(&sh.mma_done), 0);
+        }
         ptx::tc_fence_after();
         ptx::tmem_dealloc(tmem_base, C::TMEM_COLS);
     }

@@ -458,11 +458,14 @@ __device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, const W
     if (__all_sync(0xffffffffu, ptx::mbar_try_wait(bar, parity))) return true;
     return __all_sync(0xffffffffu, wait_slow(bar, parity, ctx, where));
 }
-// Bounded wait for copies that may still be in flight when a role gives up.
-__device__ __forceinline__ void drain(uint32_t bar, uint32_t parity, long long limit)
+// Wait for copies or MMAs that may still be in flight when a role gives up.  Its limit, about half a millisecond, is far
+// beyond the time that any of them takes and does not shrink with the limit of the other waits, which a test may set so
+// low that they run out while the copies they wait for are on their way.
+constexpr long long kDrainCycles = 1 << 20;
+__device__ __forceinline__ void drain(uint32_t bar, uint32_t parity)
 {
     const long long t0 = clock64();
-    while (!ptx::mbar_try_wait(bar, parity) && clock64() - t0 < limit) { }
+    while (!ptx::mbar_try_wait(bar, parity) && clock64() - t0 < kDrainCycles) { }
 }
 
 }  // namespace wfq
