@@ -96,11 +96,14 @@ typedef enum {
     WFQ_DEBUG_SKIP_GEMM_STAGE = 3,  /* operand stage (counted from 0) whose loads the first
                                        CTA of the contraction kernel does not issue (-1 =
                                        none); same purpose as WFQ_DEBUG_SKIP_INPUT_ITEM */
-    WFQ_DEBUG_GEMM_SHAPE = 4        /* 0: the library chooses the contraction's orientation and
+    WFQ_DEBUG_GEMM_SHAPE = 4,       /* 0: the library chooses the contraction's orientation and
                                        column block; else 100 * orientation (1: accumulator rows are
                                        tiles, 2: rows are output channels) + columns per unit (16 or
                                        64 for orientation 1; 16, 32, 48 or 64 for orientation 2).
                                        Results do not depend on it; for timing experiments */
+    WFQ_DEBUG_GEMM_CTAS = 5         /* 0: two per SM; else the CTAs (up to 65535) over which the contraction
+                                       deals its units, which decides how many of the last ones it cuts
+                                       into parts.  Results do not depend on it */
 } wfq_debug_option_t;
 
 /*

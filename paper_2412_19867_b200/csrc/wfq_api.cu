@@ -289,6 +289,7 @@ wfq_status_t wfq_plan_set_workspace(wfq_plan_t *plan, void *dev_ptr, size_t byte
         return WFQ_ERR_INVALID_ARG;
     wfq_status_t bs = bind_device(plan);
     if (bs != WFQ_OK) return bs;
+    plan->has_workspace = false;      // until the tensor maps describe the new buffers
     wfq::Workspace &ws = plan->ws;
     char *base = static_cast<char *>(dev_ptr);
     ws.Xq = reinterpret_cast<int8_t *>(base);
@@ -577,6 +578,7 @@ static wfq_status_t setup_host_pipeline(wfq_plan *plan)
         // same orientation of the contraction as the whole batch: identical arithmetic
         q->gemm_swap = plan->gemm_swap;
         q->gemm_bn = plan->gemm_bn;
+        q->debug_gemm_ctas = plan->debug_gemm_ctas;
         const size_t slice = align_up(q->ws.total, 1024);
         if (2 * slice > plan->ws.total) return WFQ_ERR_UNSUPPORTED;
         st = wfq_plan_set_workspace(q, reinterpret_cast<char *>(plan->ws.Xq) + s * slice, slice);
@@ -719,10 +721,18 @@ wfq_status_t wfq_plan_set_debug_option(wfq_plan_t *plan, wfq_debug_option_t opti
             if (plan->Wq)
                 plan->tmap_wq_ok = wfq::encode_tmap_bytes3d(&plan->tmap_wq, plan->Wq, g.C, g.K, g.P,
                                                            swap ? wfq::gemm_block_m() : bn);
-            if ((plan->has_workspace && !plan->tmap_xq_ok) || (plan->Wq && !plan->tmap_wq_ok)) return WFQ_ERR_CUDA;
+            if ((plan->has_workspace && !plan->tmap_xq_ok) || (plan->Wq && !plan->tmap_wq_ok)) {
+                plan->has_workspace = plan->prepared = false;
+                return WFQ_ERR_CUDA;
+            }
             plan->host_chunks = 0;      // the sub-plans of the host-buffer path copy the shape when rebuilt
             break;
         }
+        case WFQ_DEBUG_GEMM_CTAS:
+            if (value < 0 || value > 65535) return WFQ_ERR_INVALID_ARG;
+            plan->debug_gemm_ctas = (int)value;
+            if (plan->has_workspace && !(plan->has_workspace = wfq::plan_gemm_units(*plan))) return WFQ_ERR_CUDA;
+            break;
         default:
             return WFQ_ERR_INVALID_ARG;
     }

@@ -611,14 +611,13 @@ cudaError_t launch_variant(const wfq_plan &plan, int32_t *acc_dump, cudaStream_t
     a.wait_cycles = plan.wait_cycles;
     a.debug_skip_stage = plan.debug_skip_gemm_stage;
     const int MT = (a.rows + BM - 1) / BM, NT = (a.cols + BN - 1) / BN;
-    const int slots = 2 * plan.sm_count;          // two CTAs per SM
     const int units = g.P * MT * NT;
     a.whole = DUMP ? units : plan.gemm_whole;     // the debug output is not cut
     a.parts = DUMP ? 1 : plan.gemm_parts;
     a.items = a.whole + (units - a.whole) * a.parts;
     a.by_NT = plan.gemm_by_nt;
     a.by_MT = plan.gemm_by_mt;
-    const int grid = a.items < slots ? a.items : slots;
+    const int grid = a.items < plan.gemm_ctas ? a.items : plan.gemm_ctas;   // the layout above is for this grid alone
     // the filters share L2 (126 MB) with Xq, sX and Y: at most 48 MB of them are asked for early
     a.l2_prefetch_bytes = pdl ? (48LL << 20) / grid : 0;
     auto kern = gemm_dequant_kernel<BN, SWAP, DUMP, false>;
@@ -759,11 +758,14 @@ bool plan_gemm_units(wfq_plan &plan)
 {
     const Geometry &g = plan.geo;
     const int bn = plan.gemm_bn, rows = plan.gemm_swap ? g.K : g.T, cols = plan.gemm_swap ? g.T : g.K;
-    const int units = g.P * ((rows + BM - 1) / BM) * ((cols + bn - 1) / bn), slots = 2 * plan.sm_count;
-    const int rest = slots > 0 ? units % slots : 0;
+    const int units = g.P * ((rows + BM - 1) / BM) * ((cols + bn - 1) / bn);
+    int ctas = plan.debug_gemm_ctas > 0 ? plan.debug_gemm_ctas : 2 * plan.sm_count;     // two per SM
+    if (ctas < 1) ctas = 1;
+    const int rest = units % ctas;
     const int part = 16 * part_pieces(bn), parts = bn / part;
     const int cg = groups_per_chunk(g.gs, bn);
-    const bool cut = parts > 1 && rest > 0 && parts * rest <= slots && (g.G + cg - 1) / cg > 1 && cols > part;
+    const bool cut = parts > 1 && rest > 0 && parts * rest <= ctas && (g.G + cg - 1) / cg > 1 && cols > part;
+    plan.gemm_ctas = ctas;
     plan.gemm_whole = cut ? units - rest : units;
     plan.gemm_parts = cut ? parts : 1;
     plan.gemm_by_nt = FastDiv((cols + bn - 1) / bn);

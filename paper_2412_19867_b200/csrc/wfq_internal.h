@@ -177,6 +177,8 @@ struct wfq_plan {
     int gemm_bn = 64;          // columns per unit of the contraction
     int gemm_whole = 0;        // units of the contraction that are one work item each; the others are cut into
     int gemm_parts = 1;        // this many parts along their columns
+    int gemm_ctas = 0;         // CTAs that this layout of work items is for: the launch takes its grid from here
+    int debug_gemm_ctas = 0;   // WFQ_DEBUG_GEMM_CTAS
     wfq::FastDiv gemm_by_nt, gemm_by_mt;   // blocks of columns and of rows of the contraction
 
     // wfq_conv_forward_host on batches of several images: the batch is cut into chunks

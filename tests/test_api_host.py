@@ -136,6 +136,15 @@ def test_weight_bits_and_blob_size(lib):
     assert lib.wfq_plan_destroy(plan) == b.WFQ_OK
 
 
+def test_contraction_ctas_option_range(lib):
+    st, plan = _create(lib, 1, 64, 64, 8, 8, 4, 3, 32, 8)
+    assert st == b.WFQ_OK
+    for value, want in ((0, b.WFQ_OK), (1, b.WFQ_OK), (65535, b.WFQ_OK), (-1, b.WFQ_ERR_INVALID_ARG),
+                        (65536, b.WFQ_ERR_INVALID_ARG)):
+        assert lib.wfq_plan_set_debug_option(plan, b.WFQ_DEBUG_GEMM_CTAS, ctypes.c_longlong(value)) == want, value
+    lib.wfq_plan_destroy(plan)
+
+
 def test_status_strings(lib):
     seen = {b.status_string(i) for i in range(7)}
     assert len(seen) == 7 and "ok" in seen

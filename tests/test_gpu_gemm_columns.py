@@ -51,11 +51,46 @@ def test_partial_row_blocks(T):
                          sw[:, g, :K, None] * sx[:, g, None, :T] for g in range(C // gs)])
     # a product with each scale and a sum: each rounds once per group
     bound = (C // gs + 2) * 2.0 ** -24 * terms.abs().sum(0)
-    for shape in (264, 248, 232, 164, 116):      # up to 128 tiles the units of 64, 48 and 32 columns are cut into parts
+    for shape in (264, 248, 232, 164, 116):      # which units are cut is up to the number of SMs: test_cut_units
         b.wfq_plan_set_debug_option(conv.plan, b.WFQ_DEBUG_GEMM_SHAPE, shape)
         Y = conv.buffer(b.WFQ_BUF_Y).fill_(float("nan"))
         b.wfq_gemm_dequantize(conv.plan, conv._stream())
         assert ((Y[:, :, :T].double() - terms.sum(0)).abs() <= bound).all(), shape
         assert shape >= 200 or torch.isnan(Y[:, :, (T + 3) // 4 * 4:]).all()
     conv.check_status()
+    conv.close()
+
+
+@pytest.mark.parametrize("T,K", [(161, 200), (257, 72), (129, 129), (97, 264)])
+@pytest.mark.parametrize("shape,parts", [(164, 2), (264, 2), (248, 3), (232, 2)])
+def test_cut_units(shape, parts, T, K):
+    """Whole rounds of units followed by a round that is cut into parts of their columns, with ragged tiles and channels:
+    equal bit for bit to the same layer on one CTA, where nothing is cut, and nothing else of Y is written.  The CTAs are
+    given, so the coverage does not depend on the device: a last round of r units is cut if r * parts of them have
+    room, a unit has several chunks (here three groups of 64 channels, two to a chunk) and more columns than a part."""
+    import torch
+    m, C, gs = 4, 192, 64
+    gen = torch.Generator(device="cuda").manual_seed(T + K)
+    x = torch.randn((1, C, m, m * T), generator=gen, device="cuda").half()
+    conv = b.Conv(1, C, K, m, m * T, m, gs, "f16")
+    conv.prepare(torch.randn((K, C, 3, 3), generator=gen, device="cuda"))
+    b.wfq_plan_set_debug_option(conv.plan, b.WFQ_DEBUG_GEMM_SHAPE, shape)
+    b.wfq_input_transform_quantize(conv.plan, x.data_ptr(), conv._stream())
+    rows, cols, bn = (K, T, shape - 200) if shape >= 200 else (T, K, shape - 100)
+    units = conv.P * -(-rows // 128) * -(-cols // bn)
+
+    def contract(ctas):
+        b.wfq_plan_set_debug_option(conv.plan, b.WFQ_DEBUG_GEMM_CTAS, ctas)
+        Y = conv.buffer(b.WFQ_BUF_Y).fill_(float("nan"))
+        b.wfq_gemm_dequantize(conv.plan, conv._stream())
+        conv.check_status()
+        return Y.clone()
+
+    want = contract(1)
+    assert not torch.isnan(want[:, :, :T]).any()
+    cut = [c for c in range(2, units) if 0 < units % c and units % c * parts <= c]
+    for ctas in [cut[0], cut[len(cut) // 2], cut[-1], parts * units, 0]:        # several rounds, one, none in front; as chosen
+        got = contract(ctas)
+        assert torch.equal(got[:, :, :T], want[:, :, :T]), ctas
+        assert shape >= 200 or torch.isnan(got[:, :, (T + 3) // 4 * 4:]).all()
     conv.close()
