@@ -85,7 +85,7 @@ struct GemmArgs {
     int rows, cols;           // valid rows / columns: (T, K) normal, (K, T) swapped
     int cg;                   // groups per chunk
     int items;                // work items: whole units, then the parts of the units that are cut (plan_gemm_units)
-    int whole, parts;         // whole units, parts of a cut one
+    int whole;                // whole units
     FastDiv by_NT, by_MT;     // blocks of columns and of rows
     float *Y;                 // [P][K][Tp]
     int32_t *acc_dump;        // [P][T][K][G] or null
@@ -390,7 +390,7 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
 
     if (warp == 0) {
         // ---------------- TMA producer ----------------
-        // All 32 lanes walk the loop and wait together; lane 0 alone issues the copies.
+        // All 32 lanes walk the loop and wait together; an elected one issues the copies.
         // (A warp whose other lanes sit at the final block barrier while one lane works
         // gets scheduled far too rarely.)
         int stage = 0;
@@ -433,7 +433,7 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
-        // The warp stays converged; lane 0 issues every MMA and commit.  Its instructions
+        // The warp stays converged; an elected lane issues every MMA and commit.  Its instructions
         // form one dependent chain, so the descriptors are advanced with 32-bit adds and
         // the accumulate flag is a constant of the instruction.
         constexpr uint32_t dhi = ptx::smem_desc_sw128_hi();
@@ -555,9 +555,9 @@ gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         // The parts of cut units (at most one per CTA) run code of their own: a bound on the pieces inside the unrolled
         // loops keeps the compiler from interleaving them (34 layers 5 % slower, up to 13 %)
         for (int i = blockIdx.x; i < a.whole && ok; i += gridDim.x) {
-            const int r = i / a.by_NT, p = r / a.by_MT;
-            const int nt = i - r * NT, mt = r - p * MT;
-            ok = epilogue_unit<BN, SWAP, DUMP, CUT, BN / 16>(sh, tmY, a, g, ctx, ec, p, mt, nt * BN, 0, slot, sphase);
+            const Item it = item_of<BN, false>(a, i, MT, NT);
+            ok = epilogue_unit<BN, SWAP, DUMP, CUT, BN / 16>(sh, tmY, a, g, ctx, ec, it.p, it.mt, it.nt * BN, 0, slot,
+                                                             sphase);
         }
         const int tail = a.whole + (int)blockIdx.x;
         if (CUT && tail < a.items && ok) {
@@ -613,8 +613,7 @@ cudaError_t launch_variant(const wfq_plan &plan, int32_t *acc_dump, cudaStream_t
     const int MT = (a.rows + BM - 1) / BM, NT = (a.cols + BN - 1) / BN;
     const int units = g.P * MT * NT;
     a.whole = DUMP ? units : plan.gemm_whole;     // the debug output is not cut
-    a.parts = DUMP ? 1 : plan.gemm_parts;
-    a.items = a.whole + (units - a.whole) * a.parts;
+    a.items = a.whole + (units - a.whole) * plan.gemm_parts;
     a.by_NT = plan.gemm_by_nt;
     a.by_MT = plan.gemm_by_mt;
     const int grid = a.items < plan.gemm_ctas ? a.items : plan.gemm_ctas;   // the layout above is for this grid alone
@@ -622,7 +621,7 @@ cudaError_t launch_variant(const wfq_plan &plan, int32_t *acc_dump, cudaStream_t
     a.l2_prefetch_bytes = pdl ? (48LL << 20) / grid : 0;
     auto kern = gemm_dequant_kernel<BN, SWAP, DUMP, false>;
     if constexpr (BN != 16 && !DUMP)
-        if (a.parts > 1) kern = gemm_dequant_kernel<BN, SWAP, DUMP, true>;
+        if (plan.gemm_parts > 1) kern = gemm_dequant_kernel<BN, SWAP, DUMP, true>;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3(NUM_THREADS);

@@ -18,7 +18,7 @@ enum WaitId : int {
     kWaitSmemEmpty = 1,   // TMA producer waiting for a free pipeline stage
     kWaitSmemFull = 2,    // MMA issuer waiting for TMA data
     kWaitTmemEmpty = 3,   // MMA issuer waiting for a drained accumulator
-    kWaitTmemFull = 4,    // epilogue waiting for a finished accumulator
+    kWaitTmemFull = 4,    // epilogue waiting for a finished accumulator and its scales (one barrier)
     kWaitDrain = 5,       // teardown waiting for copies in flight
     kWaitScaleEmpty = 6,  // scale loader waiting for a free ring slot
     kWaitStripEmpty = 8,  // input transform: TMA producer waiting for a free strip buffer
