@@ -26,9 +26,12 @@
 //            chunk of a unit write Y[p][k][t].
 // The second CTA of the SM runs the same pipeline on other units, which hides part of the
 // hand-over latencies; the stores of Y leave through the TMA unit (rows = tiles).
-// What bounds it: a chunk of 2 x 64 columns takes an epilogue warp 541 cycles alone and 867 beside
-// the other CTA's (784 for both at the full rate of its arithmetic), and some 300 more pass between
-// chunks; 14x14 with groups of 32, 1024 tiles x 256 channels: 16 us for 75 M group sums and 50 MB.
+// What bounds it: the epilogue warps.  14x14 with groups of 32 (1024 tiles x 256 channels, F(4,3): 3.9
+// units of four chunks per CTA, 75 M group sums), this kernel launched back to back on warm operands,
+// 20.7 us from launch to launch; with clock reads in the epilogue, which cost 10 %: a chunk of 2 x 64
+// columns takes 1110 cycles (840 with one CTA per SM) and 140 pass until the next one is complete, a
+// unit's first chunk comes after 460 and handing its Y to the TMA unit takes 780; 26 k cycles, 13.5 us,
+// in all, and 0.5 us in front of them.
 // Four epilogue warps per CTA: eight, with half of the columns each, are 1 % slower (forward, ten
 // layers), and the registers for 64 sums and two blocks of 16 leave no room for more.
 // Every wait is bounded; on expiry the CTA records where, stops, drains and frees TMEM.
